@@ -1,7 +1,7 @@
 """Build the in-tree host library libchem.so (C++ host code; the CUDA kernels themselves are
 generated per mechanism and compiled for sm_103a by NVRTC at load time, see csrc/chem_host.cpp).
 
-The device source csrc/ros4_device.cuh is embedded into the library as a string so that the
+The device source (csrc/fxmath.cuh, csrc/ros4_device.cuh) is embedded into the library as a string so that the
 library is self-contained.
 """
 from __future__ import annotations
@@ -16,12 +16,13 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT_DIR, "libchem.so")
 CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-SOURCES = [os.path.join(CSRC, "chem_host.cpp"), os.path.join(CSRC, "ros4_device.cuh"),
+DEVICE = [os.path.join(CSRC, "fxmath.cuh"), os.path.join(CSRC, "ros4_device.cuh")]
+SOURCES = [os.path.join(CSRC, "chem_host.cpp"), *DEVICE,
            os.path.join(ROOT, "include", "chem.h")]
 
 
 def _embed(dst: str) -> None:
-    src = open(os.path.join(CSRC, "ros4_device.cuh")).read()
+    src = "".join(open(p).read() for p in DEVICE)
     delim = "CHEMSRC"
     assert ")" + delim not in src
     # split into chunks below the portable string-literal limit and concatenate

@@ -8,6 +8,7 @@
 #include <nvrtc.h>
 
 #include <algorithm>
+#include <array>
 #include <climits>
 #include <cmath>
 #include <cstdarg>
@@ -410,6 +411,189 @@ std::vector<int> kernel_reaction_order(const MechData& m, bool costliest_first) 
   return order;
 }
 
+constexpr long double kLn2 = 0.693147180559945309417232121458176568L;
+
+// log2 of exp(s/R - h/RT) per species without its terms a1 log2 T and -a6 / (T ln2): a polynomial in T
+double nasa_log2_g(const double* a, int i) {
+  if (i == 0) return (double)(((long double)a[6] - a[0]) / kLn2);
+  return (double)(a[i] / (i * (i + 1) * kLn2));
+}
+
+// Whether the kernels may keep rate and equilibrium constants as Q52 logarithms (|log2| < 2048) for
+// every temperature between 256 and 8192 K (fx_range): the coefficients fit their formats and no
+// sum of them, taken with its terms' magnitudes, leaves +-1900 on a grid of temperatures (the
+// functions are smooth; a mechanism that fails takes the FP64 functions).
+bool fx_mechanism(const MechData& m) {
+  if (m.sp.size() > 65535) return false;  // 16-bit indices in mk_rec
+  const double ln2 = (double)kLn2, th_max = 180000.0 * ln2;
+  for (auto& x : m.rx) {
+    if (std::fabs(x.b) > 60.0 || std::fabs(x.theta) > th_max) return false;
+    if (x.kind >= 2 && (std::fabs(x.b0) > 60.0 || std::fabs(x.theta0) > th_max)) return false;
+  }
+  std::vector<double> g(m.sp.size());
+  for (int i = 0; i <= 500; ++i) {
+    const double T = 256.0 * std::pow(32.0, i / 500.0), l2 = std::log2(T);
+    for (size_t k = 0; k < g.size(); ++k) {
+      double mx = 0;  // both ranges of the polynomials: the switch lies between two grid points
+      for (const double* a : {m.sp[k].nasa[0], m.sp[k].nasa[1]}) {
+        double c[5];
+        for (int j = 0; j < 5; ++j) c[j] = nasa_log2_g(a, j);
+        if (std::fabs(a[0]) > 60.0 || std::fabs(a[5]) > th_max) return false;
+        const bool used = (a == m.sp[k].nasa[0]) ? T < 1.02 * m.sp[k].Tmid : T > 0.98 * m.sp[k].Tmid;
+        if (!used) continue;
+        const double v = a[0] * l2 - a[5] / (T * ln2) + c[0] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4])));
+        if (!(std::fabs(v) < 1900.0)) return false;
+        if (std::fabs(v) > std::fabs(mx)) mx = v;
+      }
+      g[k] = mx;
+    }
+    for (auto& x : m.rx) {
+      double kc = 0;
+      int d = 0;
+      for (int j = 0; j < x.npr; ++j) { kc += x.pnu[j] * g[x.psp[j]]; d += x.pnu[j]; }
+      for (int j = 0; j < x.nre; ++j) { kc -= x.rnu[j] * g[x.rsp[j]]; d -= x.rnu[j]; }
+      const double kinf = (std::fabs(x.lnA) + std::fabs(x.theta) / T) / ln2 + std::fabs(x.b) * l2;
+      // low-pressure limit, [M] of 1e-300..1e30 after the floor, a Troe blend of 10^-100
+      const double k0 = x.kind >= 2 ? (std::fabs(x.lnA0) + std::fabs(x.theta0) / T) / ln2 + std::fabs(x.b0) * l2 + 334.0 : 0.0;
+      if (!(kinf + k0 + std::fabs(kc) + std::abs(d) * 20.0 < 1900.0)) return false;
+      if (x.kind >= 2 && !(kinf + 997.0 + 334.0 + std::fabs(kc) + std::abs(d) * 20.0 < 2040.0)) return false;
+    }
+  }
+  return true;
+}
+
+// Reactions per chunk of the multi-lane kernels' reaction loop: the net rates and rate constants of
+// a chunk sit in shared memory while they are gathered per species and per Jacobian entry.  A
+// multiple of the team (one reaction per lane at least) for which the rate constants fit among the
+// stage slots that are dead then; never more than the mechanism has.
+int chunk_size(int ns, int nr, int team, int stages) {
+  const int room = (std::max(stages, 3) - 1) * ns / 2;
+  const int c = std::max(team, room / team * team);
+  return std::min(std::min(c, 512), nr);
+}
+
+// both sides of at most second order: d q / d C is a coefficient times k times one concentration
+bool second_order(const ReactionData& x) {
+  int a = 0, b = 0;
+  for (int i = 0; i < x.nre; ++i) a += x.rnu[i];
+  for (int i = 0; i < x.npr; ++i) b += x.pnu[i];
+  return a <= 2 && b <= 2;
+}
+
+// The chunks' gather lists (gather_run and gather_jacobian of the device code).
+//  * mk_oseg, per chunk: runs of up to seven entries of one species, one per lane and pass; up to
+//    eight runs of a species lie next to each other within a warp and are summed by shuffles.
+//  * mk_jent, per chunk: for every lane a stream of contributions to Jacobian entries in groups of
+//    four, stored group-major.  All contributions of an entry within a chunk are one lane's, one
+//    after another; one of coefficient n stands n times.
+void emit_gather(std::ostringstream& o, const MechData& m, int team, int chunk) {
+  const int ns = (int)m.sp.size(), nr = (int)m.rx.size(), nch = (nr + chunk - 1) / chunk;
+  o << "#define CHUNK " << chunk << "\n#define NCHUNK " << nch << "\n";
+  if (team == 1) {
+    o << "#define HAS_GENERAL 0\n#define GATHER_J 0\n";
+    return;
+  }
+  bool general = false;
+  for (auto& x : m.rx) general = general || !second_order(x);
+  // the records' fields: 14 bits of entry, 9 of position, 7 of species
+  const bool gather_j = ns * ns <= 16384 && ns <= 126 && chunk <= 256;
+  o << "#define HAS_GENERAL " << (general ? 1 : 0) << "\n#define GATHER_J " << (gather_j ? 1 : 0) << "\n";
+  const int bath = ns - 1;
+  auto smap = [&](int k) { return k == bath ? 0 : k + 1; };
+  std::vector<int> segoff(1, 0), joff(1, 0);
+  std::vector<std::array<uint32_t, 4>> segs, jent;
+  for (int ch = 0; ch < nch; ++ch) {
+    const int r0 = ch * chunk, r1 = std::min(nr, r0 + chunk);
+    std::vector<std::vector<uint32_t>> by(ns);
+    std::map<int, std::vector<uint32_t>> tgt;
+    for (int r = r0; r < r1; ++r) {
+      const ReactionData& x = m.rx[r];
+      const uint32_t j = (uint32_t)(r - r0);
+      for (int i = 0; i < x.nre; ++i) by[x.rsp[i]].insert(by[x.rsp[i]].end(), x.rnu[i], j | 0x8000u);
+      for (int i = 0; i < x.npr; ++i) by[x.psp[i]].insert(by[x.psp[i]].end(), x.pnu[i], j);
+      if (!second_order(x) || !gather_j) continue;
+      for (int side = 0; side < 2; ++side) {
+        const int n = side ? x.npr : x.nre;
+        const int* sp = side ? x.psp : x.rsp;
+        const int* nu = side ? x.pnu : x.rnu;
+        for (int d = 0; d < n; ++d) {
+          // d(k prod c^nu)/d c_d = nu_d k times the one remaining concentration, if any
+          const uint32_t other = nu[d] == 2 ? (uint32_t)sp[d] : (n == 2 ? (uint32_t)sp[1 - d] : 127u);
+          auto add = [&](int row, int nurow) {
+            const int cf = nurow * nu[d] * (side ? -1 : 1), t = smap(row) * ns + smap(sp[d]);
+            const uint32_t e = (uint32_t)t | (j + (uint32_t)(side * chunk)) << 14 | other << 23 | (cf < 0 ? 1u << 31 : 0u);
+            for (int q = 0; q < std::abs(cf); ++q) tgt[t].push_back(e);
+          };
+          for (int i = 0; i < x.nre; ++i) add(x.rsp[i], -x.rnu[i]);
+          for (int i = 0; i < x.npr; ++i) add(x.psp[i], x.pnu[i]);
+        }
+      }
+    }
+    // longest species first, so that groups of runs seldom have to skip lanes to stay in a warp
+    std::vector<int> sp(ns);
+    for (int k = 0; k < ns; ++k) sp[k] = k;
+    std::stable_sort(sp.begin(), sp.end(), [&](int a, int b) { return by[a].size() > by[b].size(); });
+    const size_t warp = (size_t)std::min(team, 32), most = std::min<size_t>(8, warp);
+    const std::array<uint32_t, 4> none = {0x4000u << 16, 0x40004000u, 0x40004000u, 0x40004000u};
+    for (int k : sp) {
+      const bool atomic = by[k].size() > 7 * most;
+      for (size_t g0 = 0; g0 < by[k].size(); g0 += 7 * most) {
+        const size_t ne = std::min(by[k].size() - g0, 7 * most), nrun = (ne + 6) / 7;
+        while (segs.size() % warp + nrun > warp) segs.push_back(none);
+        for (size_t a = 0; a < nrun; ++a) {
+          uint32_t e[8] = {(uint32_t)k};
+          // after step o a lane holds the sum of min(2 o, runs to its right) runs
+          for (size_t o = 1, b = 0; o < 8; o <<= 1, ++b)
+            if (a + o < nrun) e[0] |= 0x100u << b;
+          if (a == 0) e[0] |= atomic ? 0x1000u : 0x800u;
+          for (size_t i = 0; i < 7; ++i) e[1 + i] = 7 * a + i < ne ? by[k][g0 + 7 * a + i] : 0x4000u;
+          segs.push_back({e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16, e[6] | e[7] << 16});
+        }
+      }
+    }
+    while (segs.size() % (size_t)team) segs.push_back(none);
+    segoff.push_back((int)segs.size());
+    // Jacobian entries: longest first to the lane with the shortest stream
+    std::vector<std::pair<int, int>> order;
+    for (auto& t : tgt) order.push_back({-(int)t.second.size(), t.first});
+    std::sort(order.begin(), order.end());
+    std::vector<std::vector<uint32_t>> lane(team);
+    for (auto& t : order) {
+      int best = 0;
+      for (int l = 1; l < team; ++l) if (lane[l].size() < lane[best].size()) best = l;
+      bool first = true;
+      for (uint32_t e : tgt[t.second]) {
+        lane[best].push_back(e | (first ? 0u : 1u << 30));
+        first = false;
+      }
+    }
+    size_t steps = 0;
+    for (auto& l : lane) steps = std::max(steps, l.size());
+    steps = (steps + 3) / 4;
+    for (size_t t = 0; t < steps; ++t)
+      for (auto& l : lane) {
+        std::array<uint32_t, 4> g;
+        for (size_t i = 0; i < 4; ++i) g[i] = 4 * t + i < l.size() ? l[4 * t + i] : 126u << 23;
+        jent.push_back(g);
+      }
+    joff.push_back(joff.back() + (int)steps);
+  }
+  if (jent.empty()) jent.push_back({});
+  auto table = [&](const char* name, const std::vector<std::array<uint32_t, 4>>& v) {
+    emit_array(o, "uint4", name, "[" + std::to_string(v.size()) + "]", (int)v.size(), [&](int i) {
+      return "{" + std::to_string(v[i][0]) + "u," + std::to_string(v[i][1]) + "u," + std::to_string(v[i][2]) + "u," +
+             std::to_string(v[i][3]) + "u}";
+    });
+  };
+  auto offsets = [&](const char* name, const std::vector<int>& v) {
+    emit_array(o, "int", name, "[" + std::to_string(v.size()) + "]", (int)v.size(), [&](int i) { return std::to_string(v[i]); });
+  };
+  offsets("mk_osegoff", segoff);
+  table("mk_oseg", segs);
+  offsets("mk_joff", joff);
+  table("mk_jent", jent);
+}
+
 std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, int tableau) {
   const std::vector<int> order = kernel_reaction_order(m0, !adjoint);
   MechData m = m0;
@@ -462,60 +646,23 @@ std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, 
   };
   nasa_table("mk_cp", 5, [](const double* a, int i) { return a[i]; });
   nasa_table("mk_h", 6, [](const double* a, int i) { return i < 5 ? a[i] / (i + 1) : a[5]; });
-  nasa_table("mk_s", 7, [](const double* a, int i) {
-    if (i == 0) return a[0];
-    if (i < 5) return a[i] / i;
-    return i == 6 ? a[6] : 0.0;
-  });
+  if (adjoint)
+    nasa_table("mk_s", 7, [](const double* a, int i) {
+      if (i == 0) return a[0];
+      if (i < 5) return a[i] / i;
+      return i == 6 ? a[6] : 0.0;
+    });
+  nasa_table("mk_g", 5, nasa_log2_g);
   nasa_table("mk_dcp", 4, [](const double* a, int i) { return a[i + 1] * (i + 1); });
   const std::string R = "[" + std::to_string(nr) + "]";
   const std::string RP = "[" + std::to_string(nr) + "][" + std::to_string(kMaxSide) + "]";
   emit_array(o, "int", "mk_rorig", R, nr, [&](int r) { return std::to_string(order[r]); });
-  emit_array(o, "int", "mk_kind", R, nr, [&](int r) { return std::to_string(m.rx[r].kind); });
-  emit_array(o, "double", "mk_lnA", R, nr, [&](int r) { return num(m.rx[r].lnA); });
-  emit_array(o, "double", "mk_b", R, nr, [&](int r) { return num(m.rx[r].b); });
-  emit_array(o, "double", "mk_th", R, nr, [&](int r) { return num(m.rx[r].theta); });
-  emit_array(o, "int", "mk_nre", R, nr, [&](int r) { return std::to_string(m.rx[r].nre); });
-  emit_array(o, "int", "mk_npr", R, nr, [&](int r) { return std::to_string(m.rx[r].npr); });
-  auto side_table = [&](const char* name, int ReactionData::*cnt, int (ReactionData::*arr)[kMaxSide]) {
-    o << "__device__ const int " << name << RP << " = {";
-    for (int r = 0; r < nr; ++r) {
-      o << (r ? "," : "") << "{";
-      for (int i = 0; i < kMaxSide; ++i) o << (i ? "," : "") << (i < m.rx[r].*cnt ? (m.rx[r].*arr)[i] : 0);
-      o << "}";
-    }
-    o << "};\n";
-  };
-  side_table("mk_rsp", &ReactionData::nre, &ReactionData::rsp);
-  side_table("mk_rnu", &ReactionData::nre, &ReactionData::rnu);
-  side_table("mk_psp", &ReactionData::npr, &ReactionData::psp);
-  side_table("mk_pnu", &ReactionData::npr, &ReactionData::pnu);
-  emit_array(o, "int", "mk_dnu", R, nr, [&](int r) {
-    int d = 0;
-    for (int i = 0; i < m.rx[r].npr; ++i) d += m.rx[r].pnu[i];
-    for (int i = 0; i < m.rx[r].nre; ++i) d -= m.rx[r].rnu[i];
-    return std::to_string(d);
-  });
-  // the same coefficients as doubles: the rate arithmetic reads them without an integer-to-FP64
-  // conversion (on GB300 every FP64-pipe instruction is scarce)
-  auto side_table_f = [&](const char* name, int ReactionData::*cnt, int (ReactionData::*arr)[kMaxSide]) {
-    o << "__device__ const double " << name << RP << " = {";
-    for (int r = 0; r < nr; ++r) {
-      o << (r ? "," : "") << "{";
-      for (int i = 0; i < kMaxSide; ++i) o << (i ? "," : "") << (i < m.rx[r].*cnt ? (m.rx[r].*arr)[i] : 0) << ".0";
-      o << "}";
-    }
-    o << "};\n";
-  };
-  side_table_f("mk_rnuf", &ReactionData::nre, &ReactionData::rnu);
-  side_table_f("mk_pnuf", &ReactionData::npr, &ReactionData::pnu);
-  emit_array(o, "double", "mk_dnuf", R, nr, [&](int r) {
-    int d = 0;
-    for (int i = 0; i < m.rx[r].npr; ++i) d += m.rx[r].pnu[i];
-    for (int i = 0; i < m.rx[r].nre; ++i) d -= m.rx[r].rnu[i];
-    return std::to_string(d) + ".0";
-  });
-  std::vector<int> off(nr + 1, 0), esp;
+  // rate constants as base-2 logarithms in fixed point (fxmath.cuh): {log2 A in Q52, b in Q57},
+  // {theta / ln2 in Q45, the reaction's range of third-body efficiencies}; the same of the low-pressure limits; Troe exponents times log2(e)
+  auto q = [](long double v, int n) { return std::to_string(llrintl(ldexpl(v, n))) + "LL"; };
+  const bool fx = fx_mechanism(m);
+  o << "#define MECH_FX " << (fx ? 1 : 0) << "\n";
+  std::vector<int> off(nr + 1, 0), esp;  // non-default third-body efficiencies
   std::vector<double> eval;
   for (int r = 0; r < nr; ++r) {
     off[r] = (int)esp.size();
@@ -524,8 +671,97 @@ std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, 
         if (e.second != 1.0) { esp.push_back(e.first); eval.push_back(e.second - 1.0); }
   }
   off[nr] = (int)esp.size();
+  auto fx_table = [&](const char* name, double ReactionData::*lnA, double ReactionData::*b, double ReactionData::*th) {
+    o << "__device__ const longlong2 " << name << "[" << nr << "][2] = {";
+    for (int r = 0; r < nr; ++r) {
+      const ReactionData& x = m.rx[r];
+      o << (r ? "," : "") << "{{" << (fx ? q(x.*lnA / kLn2, 52) : "0") << "," << (fx ? q(x.*b, 57) : "0") << "},{"
+        << (fx ? q(x.*th / kLn2, 45) : "0") << "," << ((long long)off[r] | (long long)off[r + 1] << 32) << "LL}}";
+    }
+    o << "};\n";
+  };
+  o << "__device__ const longlong2 mk_gq[" << ns << "][2] = {";  // a1 in Q57, -a6 / ln2 in Q45
+  for (int k = 0; k < ns; ++k) {
+    o << (k ? "," : "") << "{";
+    for (int r = 0; r < 2; ++r) {
+      const double* a = m.sp[k].nasa[r];
+      o << (r ? "," : "") << "{" << (fx ? q(a[0], 57) : "0") << "," << (fx ? q(-a[5] / kLn2, 45) : "0") << "}";
+    }
+    o << "}";
+  }
+  o << "};\n";
+  fx_table("mk_kfx", &ReactionData::lnA, &ReactionData::b, &ReactionData::theta);
+  fx_table("mk_kfx0", &ReactionData::lnA0, &ReactionData::b0, &ReactionData::theta0);
+  o << "__device__ const double mk_troe_l2[" << nr << "][3] = {";
+  for (int r = 0; r < nr; ++r) {
+    const double* t = m.rx[r].troe;
+    const bool tr = m.rx[r].kind == 3;
+    o << (r ? "," : "") << "{" << num(tr ? (double)(1.0L / (t[1] * kLn2)) : 0.0) << ","
+      << num(tr ? (double)(1.0L / (t[2] * kLn2)) : 0.0) << "," << num(tr ? (double)(t[3] / kLn2) : 0.0) << "}";
+  }
+  o << "};\n";
+  emit_gather(o, m, team, chunk_size(ns, nr, team, c.s));
+  // one record per reaction (layout: reaction_loop)
+  o << "__device__ const int4 mk_rec[" << nr << "] = {";
+  for (int r = 0; r < nr; ++r) {
+    const ReactionData& x = m.rx[r];
+    int d = 0;
+    uint32_t s6[6] = {}, fl = (uint32_t)x.nre | (uint32_t)x.npr << 2 | (uint32_t)x.kind << 4;
+    for (int i = 0; i < x.nre; ++i) { s6[i] = (uint32_t)x.rsp[i]; fl |= (uint32_t)x.rnu[i] << (13 + 2 * i); d -= x.rnu[i]; }
+    for (int i = 0; i < x.npr; ++i) { s6[3 + i] = (uint32_t)x.psp[i]; fl |= (uint32_t)x.pnu[i] << (19 + 2 * i); d += x.pnu[i]; }
+    fl |= (uint32_t)(d + 16) << 8 | (second_order(x) ? 0u : 1u) << 7;
+    o << (r ? "," : "") << "{" << (int32_t)(s6[0] | s6[1] << 16) << "," << (int32_t)(s6[2] | s6[3] << 16) << ","
+      << (int32_t)(s6[4] | s6[5] << 16) << "," << (int32_t)fl << "}";
+  }
+  o << "};\n";
+  emit_array(o, "double", "mk_lnA", R, nr, [&](int r) { return num(m.rx[r].lnA); });
+  emit_array(o, "double", "mk_b", R, nr, [&](int r) { return num(m.rx[r].b); });
+  emit_array(o, "double", "mk_th", R, nr, [&](int r) { return num(m.rx[r].theta); });
+  if (adjoint) emit_array(o, "int", "mk_kind", R, nr, [&](int r) { return std::to_string(m.rx[r].kind); });
+  if (adjoint) {  // the reverse sweep's tables, one array per field
+    emit_array(o, "int", "mk_nre", R, nr, [&](int r) { return std::to_string(m.rx[r].nre); });
+    emit_array(o, "int", "mk_npr", R, nr, [&](int r) { return std::to_string(m.rx[r].npr); });
+    auto side_table = [&](const char* name, int ReactionData::*cnt, int (ReactionData::*arr)[kMaxSide]) {
+      o << "__device__ const int " << name << RP << " = {";
+      for (int r = 0; r < nr; ++r) {
+        o << (r ? "," : "") << "{";
+        for (int i = 0; i < kMaxSide; ++i) o << (i ? "," : "") << (i < m.rx[r].*cnt ? (m.rx[r].*arr)[i] : 0);
+        o << "}";
+      }
+      o << "};\n";
+    };
+    side_table("mk_rsp", &ReactionData::nre, &ReactionData::rsp);
+    side_table("mk_rnu", &ReactionData::nre, &ReactionData::rnu);
+    side_table("mk_psp", &ReactionData::npr, &ReactionData::psp);
+    side_table("mk_pnu", &ReactionData::npr, &ReactionData::pnu);
+    emit_array(o, "int", "mk_dnu", R, nr, [&](int r) {
+      int d = 0;
+      for (int i = 0; i < m.rx[r].npr; ++i) d += m.rx[r].pnu[i];
+      for (int i = 0; i < m.rx[r].nre; ++i) d -= m.rx[r].rnu[i];
+      return std::to_string(d);
+    });
+    // the same coefficients as doubles: the rate arithmetic reads them without an integer-to-FP64
+    // conversion (on GB300 every FP64-pipe instruction is scarce)
+    auto side_table_f = [&](const char* name, int ReactionData::*cnt, int (ReactionData::*arr)[kMaxSide]) {
+      o << "__device__ const double " << name << RP << " = {";
+      for (int r = 0; r < nr; ++r) {
+        o << (r ? "," : "") << "{";
+        for (int i = 0; i < kMaxSide; ++i) o << (i ? "," : "") << (i < m.rx[r].*cnt ? (m.rx[r].*arr)[i] : 0) << ".0";
+        o << "}";
+      }
+      o << "};\n";
+    };
+    side_table_f("mk_rnuf", &ReactionData::nre, &ReactionData::rnu);
+    side_table_f("mk_pnuf", &ReactionData::npr, &ReactionData::pnu);
+  }
+  emit_array(o, "double", "mk_dnuf", R, nr, [&](int r) {
+    int d = 0;
+    for (int i = 0; i < m.rx[r].npr; ++i) d += m.rx[r].pnu[i];
+    for (int i = 0; i < m.rx[r].nre; ++i) d -= m.rx[r].rnu[i];
+    return std::to_string(d) + ".0";
+  });
   const int ne = std::max<int>(1, (int)esp.size());
-  emit_array(o, "int", "mk_effoff", "[" + std::to_string(nr + 1) + "]", nr + 1, [&](int i) { return std::to_string(off[i]); });
+  if (adjoint) emit_array(o, "int", "mk_effoff", "[" + std::to_string(nr + 1) + "]", nr + 1, [&](int i) { return std::to_string(off[i]); });
   emit_array(o, "int", "mk_effsp", "[" + std::to_string(ne) + "]", ne,
              [&](int i) { return std::to_string(i < (int)esp.size() ? esp[i] : 0); });
   emit_array(o, "double", "mk_effval", "[" + std::to_string(ne) + "]", ne,
@@ -541,32 +777,34 @@ std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, 
       << num(tr ? 1.0 / t[2] : 0.0) << "," << num(tr ? t[3] : 0.0) << "}";
   }
   o << "};\n";
-  // species -> (reaction, net nu) lists cut into segments of at most kSegLen entries for the
-  // deterministic omega gather of multi-lane teams
-  std::vector<int> gbeg(1, 0), grx, spseg(1, 0);
-  std::vector<double> gnu;
-  for (int k = 0; k < ns; ++k) {
-    std::vector<std::pair<int, int>> lst;
-    for (int r = 0; r < nr; ++r) {
-      int nu = 0;
-      for (int i = 0; i < m.rx[r].npr; ++i) if (m.rx[r].psp[i] == k) nu += m.rx[r].pnu[i];
-      for (int i = 0; i < m.rx[r].nre; ++i) if (m.rx[r].rsp[i] == k) nu -= m.rx[r].rnu[i];
-      if (nu) lst.push_back({r, nu});
+  if (adjoint) {
+    // species -> (reaction, net nu) lists cut into segments of at most kSegLen entries for the
+    // deterministic omega gather of multi-lane teams
+    std::vector<int> gbeg(1, 0), grx, spseg(1, 0);
+    std::vector<double> gnu;
+    for (int k = 0; k < ns; ++k) {
+      std::vector<std::pair<int, int>> lst;
+      for (int r = 0; r < nr; ++r) {
+        int nu = 0;
+        for (int i = 0; i < m.rx[r].npr; ++i) if (m.rx[r].psp[i] == k) nu += m.rx[r].pnu[i];
+        for (int i = 0; i < m.rx[r].nre; ++i) if (m.rx[r].rsp[i] == k) nu -= m.rx[r].rnu[i];
+        if (nu) lst.push_back({r, nu});
+      }
+      for (size_t a = 0; a < lst.size(); a += kSegLen) {
+        for (size_t b = a; b < std::min(lst.size(), a + kSegLen); ++b) { grx.push_back(lst[b].first); gnu.push_back(lst[b].second); }
+        gbeg.push_back((int)grx.size());
+      }
+      spseg.push_back((int)gbeg.size() - 1);
     }
-    for (size_t a = 0; a < lst.size(); a += kSegLen) {
-      for (size_t b = a; b < std::min(lst.size(), a + kSegLen); ++b) { grx.push_back(lst[b].first); gnu.push_back(lst[b].second); }
-      gbeg.push_back((int)grx.size());
-    }
-    spseg.push_back((int)gbeg.size() - 1);
+    const int nseg = (int)gbeg.size() - 1, nent = std::max<int>(1, (int)grx.size());
+    o << "#define NSEG " << std::max(nseg, 1) << "\n";
+    emit_array(o, "int", "mk_gseg_beg", "[" + std::to_string(nseg + 1) + "]", nseg + 1, [&](int i) { return std::to_string(gbeg[i]); });
+    emit_array(o, "int", "mk_gent_rx", "[" + std::to_string(nent) + "]", nent,
+               [&](int i) { return std::to_string(i < (int)grx.size() ? grx[i] : 0); });
+    emit_array(o, "double", "mk_gent_nu", "[" + std::to_string(nent) + "]", nent,
+               [&](int i) { return num(i < (int)gnu.size() ? gnu[i] : 0.0); });
+    emit_array(o, "int", "mk_spseg_beg", "[" + std::to_string(ns + 1) + "]", ns + 1, [&](int i) { return std::to_string(spseg[i]); });
   }
-  const int nseg = (int)gbeg.size() - 1, nent = std::max<int>(1, (int)grx.size());
-  o << "#define NSEG " << std::max(nseg, 1) << "\n";
-  emit_array(o, "int", "mk_gseg_beg", "[" + std::to_string(nseg + 1) + "]", nseg + 1, [&](int i) { return std::to_string(gbeg[i]); });
-  emit_array(o, "int", "mk_gent_rx", "[" + std::to_string(nent) + "]", nent,
-             [&](int i) { return std::to_string(i < (int)grx.size() ? grx[i] : 0); });
-  emit_array(o, "double", "mk_gent_nu", "[" + std::to_string(nent) + "]", nent,
-             [&](int i) { return num(i < (int)gnu.size() ? gnu[i] : 0.0); });
-  emit_array(o, "int", "mk_spseg_beg", "[" + std::to_string(ns + 1) + "]", ns + 1, [&](int i) { return std::to_string(spseg[i]); });
   o << kDeviceSource;
   o << "\nextern \"C\" __device__ const int chem_slots = SLOTS;\n";
   o << "extern \"C\" __device__ const int chem_tstride = TSTRIDE;\n";
@@ -708,15 +946,16 @@ struct chem_mech {
 
 namespace {
 
-// shared-memory slots of one cell; mirrors the OFF_* layout of ros4_device.cuh: A, Y, U1, YT,
-// U2..Us, [F0], six per-species arrays, the packed permutation (and pivots with one lane per
-// cell), 24 reduction slots
+// shared-memory slots of one cell; mirrors the OFF_* layout of ros4_device.cuh: A, Y, YT, U1..Us, [F0], five per-species arrays, the packed permutation (and pivots with one lane per
+// cell), a chunk's net rates and, where they don't fit elsewhere, rate constants, 24 reduction slots
 int slots_for(const MechData& m, int tableau, int team) {
   const int ns = (int)m.sp.size();
   const RosCoefficients c = ros_coefficients(tableau);
   const int packed = (ns + 1) / 2;
-  // stage slots: at least three after the stage argument (the Jacobian assembly aliases them)
-  return ns * ns + (8 + std::max(c.s, 3) + (needs_f0(c) ? 1 : 0)) * ns + packed * (team == 1 ? 2 : 1) + 24;
+  const int stages = std::max(c.s, 3);  // the Jacobian assembly aliases three
+  const int chunk = team == 1 ? 0 : chunk_size(ns, (int)m.rx.size(), team, c.s);
+  return ns * ns + (7 + stages + (needs_f0(c) ? 1 : 0)) * ns + packed * (team == 1 ? 2 : 1) +
+         (2 * chunk <= (stages - 1) * ns ? 1 : 3) * chunk + 24;
 }
 
 // distance in doubles between consecutive teams' slots (TSTRIDE of ros4_device.cuh): sub-warp

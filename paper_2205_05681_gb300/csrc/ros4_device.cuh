@@ -43,6 +43,13 @@
 #define R_OVER_PATM (8314.462618 / 101325.0)
 #define PATM_OVER_R (101325.0 / 8314.462618)
 #define LN10 2.302585092994046
+#define LN2 0.6931471805599453
+#define LOG10_2 0.30102999566398120
+#define LOG2_10 3.3219280948873623
+#define LOG2_PATM_R 3.60722334318630807
+// the same and log2(1e-300) in Q52
+#define FX_LOG2_PATM_R 16245489704216012LL
+#define FX_LOG2_1EM300 (-4488190239085892024LL)
 
 #define ST_OK 0
 #define ST_MAX_STEPS 1
@@ -75,36 +82,35 @@
 // in one SM's shared memory:
 // * f at a stage argument overwrites the argument (OFF_F = OFF_YT): the argument is dead once
 //   the concentrations and thermo are formed from it;
-// * the three per-species arrays only the Jacobian assembly uses alias YT, U2, U3, which are
-//   dead while the Jacobian is formed (it is the first thing a step attempt computes); the
-//   chain rule writes JT over DOMT and BE over BK in place;
+// * what only the Jacobian assembly uses aliases YT and the stage vectors, which are dead while the
+//   Jacobian is formed (it is the first thing a step attempt computes): d omega/dT in YT, B_k in the
+//   last stage slot, the rate constants of a chunk of reactions (OFF_KF) from U1 on, and, after the
+//   reactions, f(y) in U1 and AL in U2; the chain rule writes JT over DOMT and BE over BK in place;
 // * the LU keeps 1/U_kk on the diagonal of A, and the row permutation is packed two ints per
 //   slot (the single-lane layout also keeps the pivot sequence).
 #define OFF_A 0
 #define OFF_Y (OFF_A + NEQ * NEQ)
-#define OFF_U1 (OFF_Y + NEQ)
-#define OFF_YT (OFF_U1 + NEQ)
+#define OFF_YT (OFF_Y + NEQ)
 #define OFF_F OFF_YT
-#define OFF_U2 (OFF_YT + NEQ)
+#define OFF_U1 (OFF_YT + NEQ)
+#define OFF_U2 (OFF_U1 + NEQ)
 #define OFF_U3 (OFF_U2 + NEQ)
 #define OFF_U4 (OFF_U3 + NEQ)
-// at least three stage slots after the stage argument (YT, U2, U3): the Jacobian assembly's
-// three per-species arrays alias them (a two-stage method has no U3 of its own)
+// at least three stage slots (the Jacobian assembly uses the first two and the last)
 #define NSTG (RS > 3 ? RS : 3)
 #if NEED_F0
-#define OFF_F0 (OFF_U2 + (NSTG - 1) * NEQ)  // f(y) kept for a later stage whose argument is y itself
+#define OFF_F0 (OFF_U1 + NSTG * NEQ)  // f(y) kept for a later stage whose argument is y itself
 #define OFF_C (OFF_F0 + NEQ)
 #else
-#define OFF_C (OFF_U2 + (NSTG - 1) * NEQ)
+#define OFF_C (OFF_U1 + NSTG * NEQ)
 #endif
 #define OFF_CP (OFF_C + NS)
 #define OFF_HRT (OFF_CP + NS)
-#define OFF_EX (OFF_HRT + NS)
-#define OFF_IEX (OFF_EX + NS)
-#define OFF_OM (OFF_IEX + NS)
+#define OFF_G (OFF_HRT + NS)  // log2 exp(s/R - h/RT): Q52 integers, doubles outside fx_range
+#define OFF_OM (OFF_G + NS)
 #define OFF_DOMT OFF_YT
-#define OFF_BK (OFF_DOMT + NS)
-#define OFF_AL (OFF_BK + NS)
+#define OFF_BK (OFF_U1 + (NSTG - 1) * NEQ)
+#define OFF_AL OFF_U2
 #define OFF_JT OFF_DOMT
 #define OFF_BE OFF_BK
 #define PACKED_INTS(n) (((n) + 1) / 2)
@@ -114,8 +120,29 @@
 #else
 #define OFF_PERM (OFF_OM + NS)
 #endif
-#define OFF_RED (OFF_PERM + PACKED_INTS(NEQ))
+// net rates of a chunk of CHUNK reactions, and their rate constants (k_f, then k_r): where they fit
+// among the dead stage slots, else behind the net rates
+#define OFF_Q (OFF_PERM + PACKED_INTS(NEQ))
+#if TEAM == 1
+#define OFF_RED OFF_Q
+#elif 2 * CHUNK <= (NSTG - 1) * NEQ
+#define OFF_KF OFF_U1
+#define OFF_RED (OFF_Q + CHUNK)
+#else
+#define OFF_KF (OFF_Q + CHUNK)
+#define OFF_RED (OFF_Q + 3 * CHUNK)
+#endif
 #define SLOTS (OFF_RED + 24)
+// lanes that share a row (column) of the matrix in the Jacobian's row and column sums, and the row
+// count rounded up so that whole warps take part in their shuffles
+#if TEAM > 1 && TEAM >= 4 * NS
+#define RSPLIT 4
+#elif TEAM > 1 && TEAM >= 2 * NS
+#define RSPLIT 2
+#else
+#define RSPLIT 1
+#endif
+#define NS_PAD ((NS + TEAM / RSPLIT - 1) / (TEAM / RSPLIT) * (TEAM / RSPLIT))
 // distance between consecutive teams' slots: for sub-warp teams padded to TEAM (mod 16) doubles,
 // so that the teams of a half-warp reading the same offset of their arrays use disjoint banks
 #if SUBWARP
@@ -123,7 +150,7 @@
 #else
 #define TSTRIDE SLOTS
 #endif
-#define UOFF(i) ((i) == 0 ? OFF_U1 : OFF_U2 + ((i) - 1) * NEQ)
+#define UOFF(i) (OFF_U1 + (i) * NEQ)
 
 // Per-cell cache of the W-method's factorised iteration matrix (chem_int_opts.jac_cache, global
 // memory, one contiguous block per cell whatever the launch configuration): the N x N factors with
@@ -176,6 +203,29 @@ struct Team {
   __device__ __forceinline__ double& invd(int k) const { return A(k, k); }
 };
 
+extern __shared__ double smem[];
+
+__device__ __forceinline__ Team make_team() {
+  Team tm;
+#if TEAM == 1
+  tm.base = smem + threadIdx.x;
+  tm.tl = 0;
+#elif TEAM <= 32
+  tm.base = smem + (threadIdx.x / TEAM) * TSTRIDE;
+  tm.tl = threadIdx.x & (TEAM - 1);
+#else
+  tm.base = smem;
+  tm.tl = threadIdx.x;
+#endif
+  return tm;
+}
+
+// The parts of a step attempt are functions of their own, called out of line: inlined into every place
+// that uses them the integrator was 480 to 780 KB of instructions, far beyond the SM's instruction
+// caches, and spent most of its time fetching them.  They find the team's shared memory
+// themselves (a pointer argument would lose its address space).
+#define OUTLINE __device__ __noinline__
+
 // sum over the team; every lane gets the same bits (butterfly with commutative adds)
 __device__ __forceinline__ double team_sum(const Team& tm, double v) {
 #if TEAM == 1
@@ -218,6 +268,33 @@ __device__ __forceinline__ double team_max(const Team& tm, double v) {
 #endif
 }
 
+// two sums over the team in one reduction
+__device__ __forceinline__ void team_sum2(const Team& tm, double& a, double& b) {
+#if TEAM > 1
+  const unsigned msk = team_mask();
+#pragma unroll
+  for (int o = XOR0; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(msk, a, o);
+    b += __shfl_xor_sync(msk, b, o);
+  }
+#if TEAM > 32
+  double* red = &tm.base[OFF_RED];
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) {
+    red[threadIdx.x >> 5] = a;
+    red[TEAM / 32 + (threadIdx.x >> 5)] = b;
+  }
+  __syncthreads();
+  a = b = 0.0;
+  for (int w = 0; w < TEAM / 32; ++w) {
+    a += red[w];
+    b += red[TEAM / 32 + w];
+  }
+  __syncthreads();
+#endif
+#endif
+}
+
 // any-lane flag over the team
 __device__ __forceinline__ bool team_any(const Team& tm, bool f) {
 #if TEAM == 1
@@ -238,6 +315,13 @@ __device__ __forceinline__ void scatter_add(double* p, double v) {
 #endif
 }
 
+// sum over the RSPLIT adjacent lanes of a row
+__device__ __forceinline__ double rsplit_sum(double v) {
+#pragma unroll
+  for (int o = RSPLIT / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // |x| as an order-preserving integer (integer pipe instead of the FP64 pipe)
 __device__ __forceinline__ long long abs_key(double x) {
   return __double_as_longlong(x) & 0x7fffffffffffffffLL;
@@ -245,33 +329,62 @@ __device__ __forceinline__ long long abs_key(double x) {
 
 // ------------------------------------------------------------------------------ thermo + C
 
-// Concentrations, thermo per species and mixture sums for state y (slot OFF_Y or OFF_YT).
-// Returns V; writes C, cp, h/RT, exp(s/R - h/RT), its inverse and (WJ) dcp/dT.
+// Concentrations, thermo per species and mixture sums for state y (slot OFF_Y or OFF_YT): writes C,
+// cp, h/RT, log2 exp(s/R - h/RT) and (WJ) the sum of n dcp/dT.
 struct CellScalars {
-  double T, invT, lnT, V, cpm, dcpm;  // cpm = sum n_k cp_k / R, dcpm = sum n_k dcp_k/dT / R
+  double T, invT, V, cpm, dcpm;  // cpm = sum n_k cp_k / R, dcpm = sum n_k dcp_k/dT / R
+  double l2T;                    // log2 T
+  fx_i64 l2Tq, iTq;              // log2 T in Q59 and 1/T in Q71 (fx only)
+  bool fx;                       // logarithms of the rate constants in fixed point
 };
 
-// mass closure: n_bath = (1 - sum_k W_k n_k) / W_bath; n_tot = sum of all moles; V = n_tot R T/P
-__device__ __forceinline__ void closure_scalars(double T, double P, double wsum, double nsum, double* out) {
-  const double nb = (1.0 - wsum) * mk_invW[BATH];
-  const double V = (nsum + nb) * R_U * T / P;
-  out[0] = 1.0 / T;
-  out[1] = log(T);
-  out[2] = nb;
-  out[3] = V;
-  out[4] = 1.0 / V;
+// Where the fixed-point logarithms hold: 1/T < 2^-8 fits Q71 and log2 T < 13 fits Q59.  MECH_FX says
+// that the mechanism's own numbers keep every logarithm below 1900 (of 2048) over this range;
+// temperatures outside of it (or NaN) take the FP64 functions.
+__device__ __forceinline__ bool fx_range(double T) { return MECH_FX && T > 256.0 && T < 8192.0; }
+
+// mass closure: n_bath = (1 - sum_k W_k n_k) / W_bath; n_tot = sum of all moles; V = n_tot R T/P,
+// 1/V = (P/RT) / n_tot
+__device__ __forceinline__ void closure_scalars(const Team& tm, double T, double invT, double P, double wsum,
+                                                double nsum, double& nb, double& V, double& invV) {
+  nb = (1.0 - wsum) * mk_invW[BATH];
+  const double nt = nsum + nb;
+#if TEAM == 1
+  const double rn = fx_rcp(nt), rP = fx_rcp(P);
+#else
+  // two lanes take the two reciprocals at once
+  const double r = fx_rcp((tm.tl & 1) ? P : nt);
+  const unsigned msk = team_mask();
+  const double rn = __shfl_sync(msk, r, 0, WL), rP = __shfl_sync(msk, r, 1, WL);
+#endif
+  V = nt * (R_U * T) * rP;
+  invV = rn * (P * invT * INV_R_U);
 }
 
 template <bool WJ>
 __device__ __forceinline__ void thermo_conc(const Team& tm, int oy, double P, CellScalars& cs) {
   const double T = tm.at(oy, 0);
-  double sc[5];
+  cs.T = T;
+  cs.fx = fx_range(T);
+  if (cs.fx) {
+    const int e = fx_exponent(T);  // 8 .. 12
+    const fx_u64 x = fx_rcp_mant(fx_mant(T));
+    cs.iTq = (fx_i64)(x >> (e - 8));
+    cs.invT = fx_as_double(((fx_u64)(1021 - e) << 52) + ((x + 0x200) >> 10));
+    cs.l2Tq = ((fx_i64)e << 59) + (fx_log2_mant(fx_mant(T)) >> 3);
+    cs.l2T = fx_to_double(cs.l2Tq, 59);
+  } else {
+    cs.invT = 1.0 / T;
+    cs.l2T = log2(T);
+  }
+  const double invT = cs.invT, l2T = cs.l2T;
+  double nb, V, invV;
+  // the closure's sums: by the last warp alone (it holds the fewest species), while the others
+  // begin with the thermo polynomials
 #if TEAM > 32
-  // one lane computes the cell's scalars (divisions, log) and shares them: every extra warp
-  // repeating them would pay full warp-level FP64 pipe time
-  if (tm.tl < 32) {
+  if (tm.tl >= TEAM - 32) {
     double wsum = 0.0, nsum = 0.0;
-    for (int k = tm.tl; k < NS - 1; k += 32) {
+    for (int k = tm.tl - (TEAM - 32); k < NS - 1; k += 32) {
       const double n = tm.at(oy, 1 + k);
       wsum += mk_W[k] * n;
       nsum += n;
@@ -281,54 +394,71 @@ __device__ __forceinline__ void thermo_conc(const Team& tm, int oy, double P, Ce
       wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
       nsum += __shfl_xor_sync(0xffffffffu, nsum, o);
     }
-    if (tm.tl == 0) {
-      closure_scalars(T, P, wsum, nsum, sc);
-      for (int i = 0; i < 5; ++i) tm.base[OFF_RED + 16 + i] = sc[i];
+    closure_scalars(tm, T, invT, P, wsum, nsum, nb, V, invV);
+    if (tm.tl == TEAM - 1) {
+      tm.base[OFF_RED + 18] = nb;
+      tm.base[OFF_RED + 19] = V;
+      tm.base[OFF_RED + 20] = invV;
     }
   }
-  __syncthreads();
-  for (int i = 0; i < 5; ++i) sc[i] = tm.base[OFF_RED + 16 + i];
 #else
-  double wsum = 0.0, nsum = 0.0;
-  for (int k = tm.tl; k < NS - 1; k += TEAM) {
-    const double n = tm.at(oy, 1 + k);
-    wsum += mk_W[k] * n;
-    nsum += n;
+  {
+    double wsum = 0.0, nsum = 0.0;
+    for (int k = tm.tl; k < NS - 1; k += TEAM) {
+      const double n = tm.at(oy, 1 + k);
+      wsum += mk_W[k] * n;
+      nsum += n;
+    }
+    team_sum2(tm, wsum, nsum);
+    closure_scalars(tm, T, invT, P, wsum, nsum, nb, V, invV);
   }
-  wsum = team_sum(tm, wsum);
-  nsum = team_sum(tm, nsum);
-  closure_scalars(T, P, wsum, nsum, sc);
 #endif
-  const double invT = sc[0], lnT = sc[1], nb = sc[2], V = sc[3], invV = sc[4];
-  double cpm = 0.0, dcpm = 0.0;
+  double cpm = 0.0, dcpm = 0.0, cpb = 0.0, dcpb = 0.0;
   for (int k = tm.tl; k < NS; k += TEAM) {
-    const double n = k < NS - 1 ? tm.at(oy, 1 + k) : nb;
-    tm.at(OFF_C, k) = n * invV;
+    const double n = k < NS - 1 ? tm.at(oy, 1 + k) : 0.0;
     const int r = T < mk_Tmid[k] ? 0 : 1;
     const double* c = mk_cp[k][r];
     const double* hh = mk_h[k][r];
-    const double* s = mk_s[k][r];
+    const double* g = mk_g[k][r];
     const double cp = c[0] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4])));
     const double hRT = hh[0] + T * (hh[1] + T * (hh[2] + T * (hh[3] + T * hh[4]))) + hh[5] * invT;
-    const double sR = s[0] * lnT + s[6] + T * (s[1] + T * (s[2] + T * (s[3] + T * s[4])));
+    // log2 exp(s/R - h/RT): the large terms a1 log2 T and -a6/(T ln2) in fixed point, exact to 2^-52
+    const double lg = g[0] + T * (g[1] + T * (g[2] + T * (g[3] + T * g[4])));
+    if (cs.fx) {
+      const longlong2 gq = mk_gq[k][r];
+      const fx_i64 G = fx_from_double(lg, 52) + fx_mulhi_s(gq.x, cs.l2Tq) + fx_mulhi_s(gq.y, cs.iTq);
+      tm.at(OFF_G, k) = fx_as_double((fx_u64)G);
+    } else {
+      tm.at(OFF_G, k) = lg + c[0] * l2T - hh[5] * invT * (1.0 / LN2);
+    }
     tm.at(OFF_CP, k) = cp;
     tm.at(OFF_HRT, k) = hRT;
-    const double ex = exp(sR - hRT);
-    tm.at(OFF_EX, k) = ex;
-    tm.at(OFF_IEX, k) = 1.0 / ex;
     cpm += n * cp;
+    if (k == BATH) cpb = cp;
     if (WJ) {
       const double* d = mk_dcp[k][r];
       const double dcp = d[0] + T * (d[1] + T * (d[2] + T * d[3]));
       dcpm += n * dcp;
+      if (k == BATH) dcpb = dcp;
     }
   }
-  cs.T = T;
-  cs.invT = invT;
-  cs.lnT = lnT;
+#if TEAM > 32
+  __syncthreads();
+  nb = tm.base[OFF_RED + 18];
+  V = tm.base[OFF_RED + 19];
+  invV = tm.base[OFF_RED + 20];
+#endif
+  cpm += nb * cpb;  // the bath's lane
+  if (WJ) dcpm += nb * dcpb;
+  for (int k = tm.tl; k < NS; k += TEAM) tm.at(OFF_C, k) = (k < NS - 1 ? tm.at(oy, 1 + k) : nb) * invV;
   cs.V = V;
-  cs.cpm = team_sum(tm, cpm);
-  if (WJ) cs.dcpm = team_sum(tm, dcpm);
+  if (WJ) {
+    team_sum2(tm, cpm, dcpm);
+    cs.dcpm = dcpm;
+  } else {
+    cpm = team_sum(tm, cpm);
+  }
+  cs.cpm = cpm;
   tsync();
 }
 
@@ -338,168 +468,399 @@ __device__ __forceinline__ void thermo_conc(const Team& tm, int oy, double P, Ce
 __device__ __forceinline__ double dneg(double x) {
   return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ULL);
 }
-// nu * x for an integer stoichiometric coefficient nu (nuf = nu as a double): no FP64
-// instruction when |nu| = 1, the common case.  The adjoint module keeps the multiply (its
-// kernels measured faster with it); the results are the same bits either way.
-__device__ __forceinline__ double nu_times(int nu, double nuf, double x) {
-#if defined(CHEM_ADJOINT)
-  return nuf * x;
-#else
+// nu * x for an integer stoichiometric coefficient nu: no FP64 instruction when |nu| = 1, the
+// common case
+__device__ __forceinline__ double nu_times(int nu, double x) {
   if (nu == 1) return x;
   if (nu == -1) return dneg(x);
-  return nuf * x;
-#endif
+  return (double)nu * x;
 }
 
 // species index -> row/column of the state matrix: species 0..NS-2 -> 1..NS-1, bath -> 0
 __device__ __forceinline__ int smap(int k) { return k == BATH ? 0 : k + 1; }
 
+// Rate constants of one reaction and their derivatives: k_f and k_r (without the [M] factor of a
+// THIRD reaction), d ln k_f / dT at constant C, d ln k_f / d[M], d ln K_c / dT is the caller's.
+struct Rate {
+  double kf, kr, dlT, dlM;
+};
+
+// FP64 form, for temperatures, ln A values or falloff blends outside the fixed-point range; lKc is
+// log2 K_c.  Kept out of line: the normal path never comes here.
+template <bool WJ>
+__device__ __noinline__ void rate_fp(int r, int kind, double T, double invT, double l2T, double lA, double M,
+                                     double lKc, Rate* out) {
+  const double lnT = l2T * LN2;
+  const double kinf = exp(lA + mk_b[r] * lnT - mk_th[r] * invT);
+  double kf = kinf;
+  double dlkf_dT = 0.0, dlkf_dM = 0.0;
+  if (WJ) dlkf_dT = (mk_b[r] + mk_th[r] * invT) * invT;
+  if (kind >= LIND) {
+    const double k0 = exp(mk_lnA0[r] + mk_b0[r] * lnT - mk_th0[r] * invT);
+    double Pr = k0 * M / kinf;
+    bool floored = false;
+    if (Pr < 1e-300) { Pr = 1e-300; floored = true; }
+    double F = 1.0, dlF_dlPr = 0.0, dlF_dT = 0.0;
+    if (kind == TROE) {
+      const double a = mk_troe[r][0];
+      const double e3 = exp(-T * mk_troe[r][1]);
+      const double e1 = exp(-T * mk_troe[r][2]);
+      const double T2 = mk_troe[r][3];
+      const double e2 = T2 > 0.0 ? exp(-T2 * invT) : 0.0;
+      const double Fc = (1.0 - a) * e3 + a * e1 + e2;
+      const double lFc = log10(Fc);
+      const double n = 0.75 - 1.27 * lFc;
+      const double x = log10(Pr) + (-0.4 - 0.67 * lFc);
+      const double id = 1.0 / (n - 0.14 * x);
+      const double f1 = x * id;
+      const double den = 1.0 / (1.0 + f1 * f1);
+      F = exp(lFc * den * LN10);
+      if (WJ) {
+        const double g2 = 2.0 * lFc * f1 * den * den;  // -d log10F / d f1
+        if (!floored) dlF_dlPr = -g2 * n * id * id;
+        const double dFc = -(1.0 - a) * mk_troe[r][1] * e3 - a * mk_troe[r][2] * e1 +
+                           (T2 > 0.0 ? T2 * invT * invT * e2 : 0.0);
+        const double df1_dlFc = (-0.67 * n + 1.27 * x) * id * id;
+        dlF_dT = (den - g2 * df1_dlFc) * dFc / Fc;
+      }
+    }
+    kf = kinf * (Pr / (1.0 + Pr)) * F;
+    if (WJ) {
+      const double g = floored ? 0.0 : 1.0 / (1.0 + Pr) + dlF_dlPr;
+      const double dlk0 = (mk_b0[r] + mk_th0[r] * invT) * invT;
+      dlkf_dM = g / M;
+      dlkf_dT = dlkf_dT + g * (dlk0 - dlkf_dT) + dlF_dT;
+    }
+  }
+  out->kf = kf;
+  out->kr = kf * exp2(-lKc);
+  out->dlT = dlkf_dT;
+  out->dlM = dlkf_dM;
+}
+
+// Fixed-point form: log2 k in Q52 as ln A / ln2 + b log2 T - (theta / ln2) / T, the falloff blend and
+// the equilibrium constant added as logarithms, one fx_exp2 for k_f and one for k_r.  An FP64
+// exp() per reaction and the products of species' exponentials for k_r took 300 + 80 clocks of an
+// SM per warp, the two integer exponentials take 60.  Returns false where the values leave the
+// fixed-point range.
+template <bool WJ>
+__device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, const longlong2 k1, fx_i64 th,
+                                        const double* __restrict__ lA_ext, double M, fx_i64 lKc, Rate* out) {
+  fx_i64 lk = k1.x;
+  if (lA_ext) {
+    const double lA = *lA_ext;
+    if (!(fabs(lA) < 500.0)) return false;
+    lk = fx_mulhi_s(fx_from_double(lA, 54), 0x5c551d94ae0bf85eLL);  // Q54 x Q62: log2 A in Q52
+  }
+  lk += fx_mulhi_s(k1.y, cs.l2Tq) - fx_mulhi_s(th, cs.iTq);
+  if (WJ) {
+    out->dlT = (mk_b[r] + mk_th[r] * cs.invT) * cs.invT;
+    out->dlM = 0.0;
+  }
+  if (kind < LIND) {
+    out->kf = fx_exp2(lk);
+    out->kr = fx_exp2(lk - lKc);
+    return true;
+  }
+  // log2 Pr = log2 k0 + log2 [M] - log2 k_inf, floored at 1e-300
+  const longlong2 k2 = mk_kfx0[r][0];
+  const fx_i64 lfl = FX_LOG2_1EM300;
+  fx_i64 lPr = lfl;
+  bool floored = true;
+  if (fx_normal_pos(M)) {
+    const fx_i64 l = k2.x + fx_mulhi_s(k2.y, cs.l2Tq) - fx_mulhi_s(mk_kfx0[r][1].x, cs.iTq) + fx_log2(M) - lk;
+    if (l >= lfl) { lPr = l; floored = false; }
+  }
+  const double g1 = fx_rcp(1.0 + fx_exp2(lPr));  // 1 / (1 + Pr)
+  lk += lPr;
+  double dlF_dlPr = 0.0, dlF_dT = 0.0;
+  if (kind == TROE) {
+    const double a = mk_troe[r][0];
+    const double* t = mk_troe_l2[r];  // log2(e) / T***, log2(e) / T*, log2(e) T**
+    const double T = cs.T, invT = cs.invT;
+    const double e3 = fx_exp2(-fx_from_double(T * t[0], 52));
+    const double e1 = fx_exp2(-fx_from_double(T * t[1], 52));
+    double Fc = (1.0 - a) * e3 + a * e1;
+    double e2 = 0.0;
+    if (t[2] > 0.0) {
+      e2 = fx_exp2(-fx_from_double(t[2] * invT, 52));
+      Fc += e2;
+    }
+    if (!fx_normal_pos(Fc)) return false;
+    const double lFc = fx_log2_d(Fc) * LOG10_2;
+    const double n = 0.75 - 1.27 * lFc;
+    const double x = fx_to_double(lPr, 52) * LOG10_2 + (-0.4 - 0.67 * lFc);
+    const double id = fx_rcp(n - 0.14 * x);
+    const double f1 = x * id;
+    const double den = fx_rcp(1.0 + f1 * f1);
+    const double lF = lFc * den;
+    if (!(fabs(lF) < 100.0)) return false;
+    lk += fx_from_double(lF * LOG2_10, 52);
+    if (WJ) {
+      const double g2 = 2.0 * lF * f1 * den;  // -d log10F / d f1
+      const double id2 = id * id;
+      if (!floored) dlF_dlPr = -g2 * n * id2;
+      double dFc = -(1.0 - a) * mk_troe[r][1] * e3 - a * mk_troe[r][2] * e1;
+      if (t[2] > 0.0) dFc += mk_troe[r][3] * invT * invT * e2;
+      const double df1_dlFc = (-0.67 * n + 1.27 * x) * id2;
+      dlF_dT = (den - g2 * df1_dlFc) * dFc * fx_rcp(Fc);
+    }
+  }
+  out->kf = fx_exp2(lk) * g1;
+  out->kr = fx_exp2(lk - lKc) * g1;
+  if (WJ) {
+    const double g = floored ? 0.0 : g1 + dlF_dlPr;
+    const double dlk0 = (mk_b0[r] + mk_th0[r] * cs.invT) * cs.invT;
+    out->dlM = floored ? 0.0 : g * fx_rcp(M);
+    out->dlT = out->dlT + g * (dlk0 - out->dlT) + dlF_dT;
+  }
+  return true;
+}
+
+#if TEAM > 1
+// dst[k] += sum_r nu_kr q_r over a chunk's reactions (their values in OFF_Q), without shared-memory
+// atomics (a compare-and-swap loop per FP64 add: 140 clocks, and as much again for every lane that
+// hits the same species).  A lane sums a run of up to seven entries of one species (a coefficient n
+// stands n times); the runs of a species lie in neighbouring lanes and are added by shuffles, and
+// the first lane stores.  A run is one 16-byte record: species (8 bits), add the value of the lane
+// 1, 2, 4 further (bits 8..10), store (11), by an atomic (12: more than eight runs), then seven
+// entries of position (9 bits) and sign (bit 15); bit 14: none.
+__device__ __forceinline__ void gather_run(const Team& tm, const uint4 g, int dst) {
+  const unsigned e[7] = {g.x >> 16, g.y & 0xffff, g.y >> 16, g.z & 0xffff, g.z >> 16, g.w & 0xffff, g.w >> 16};
+  double q[7];
+#pragma unroll
+  for (int i = 0; i < 7; ++i) q[i] = tm.at(OFF_Q, e[i] & 0x1ff);
+#pragma unroll
+  for (int i = 0; i < 7; ++i) {
+    q[i] = (e[i] & 0x8000u) ? dneg(q[i]) : q[i];
+    q[i] = (e[i] & 0x4000u) ? 0.0 : q[i];
+  }
+  double v = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + q[6]);
+  const unsigned msk = team_mask();
+#pragma unroll
+  for (int o = 1; o < 8 && o < WL; o <<= 1) {
+    const double w = __shfl_down_sync(msk, v, o, WL);
+    if (g.x & (256u << (o >> 1))) v += w;
+  }
+  double* p = &tm.at(dst, g.x & 255u);
+  if (g.x & 0x1000u) atomicAdd(p, v);
+  else if (g.x & 0x800u) *p += v;
+}
+__device__ __forceinline__ void gather_species(const Team& tm, int ch, const uint4 first, int dst) {
+  const int n = mk_osegoff[ch + 1] - mk_osegoff[ch];  // a multiple of TEAM
+  gather_run(tm, first, dst);
+  for (int sg = tm.tl + TEAM; sg < n; sg += TEAM) gather_run(tm, mk_oseg[mk_osegoff[ch] + sg], dst);
+}
+
+#if GATHER_J
+// A[row][col] += sum of +-k x concentration over the chunk's contributions (rate constants in
+// OFF_KF): one FMA each, every entry owned by one lane.  Four contributions come in one 16-byte
+// load, issued a group ahead: entry (14 bits), position of k (9), species of the factor (7; 126:
+// none, 127: factor one), same entry as the previous contribution (1), negative (1).
+__device__ __forceinline__ void gather_jacobian(const Team& tm, int ch) {
+  const uint4* ent = mk_jent + (long long)mk_joff[ch] * TEAM + tm.tl;
+  const int n = mk_joff[ch + 1] - mk_joff[ch];
+  double last = 0.0;
+  uint4 nx = n > 0 ? ent[0] : make_uint4(0, 0, 0, 0);
+  for (int t = 0; t < n; ++t) {
+    const unsigned e[4] = {nx.x, nx.y, nx.z, nx.w};
+    if (t + 1 < n) nx = ent[(t + 1) * TEAM];
+    double a[4], k[4], c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int sp = (e[i] >> 23) & 127;
+      a[i] = tm.at(OFF_A, e[i] & 0x3fff);
+      k[i] = tm.at(OFF_KF, (e[i] >> 14) & 511);
+      c[i] = sp >= 126 ? 1.0 : tm.at(OFF_C, sp);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const double kk = (e[i] >> 31) ? dneg(k[i]) : k[i];
+      const double v = fma(kk, c[i], (e[i] & 0x40000000u) ? last : a[i]);
+      last = v;
+      if (((e[i] >> 23) & 127) != 126) tm.at(OFF_A, e[i] & 0x3fff) = v;
+    }
+  }
+}
+#endif
+#endif
+
 // Net production rates omega (slot OFF_OM, zeroed by the caller) and, with WJ, the reaction
 // part of the Jacobian: A[smap(k)][smap(j)] += d omega_k / d C_j (without the default-
 // efficiency third-body part, which is collected per species in OFF_BK), d omega_k/dT at
 // constant C in OFF_DOMT.  The caller zeroes A, OFF_DOMT and OFF_BK.
+// A reaction's indices and coefficients come in one 16-byte record: six species (16 bits each),
+// then nre, npr, kind (2 bits each), dnu + 16 (5 bits, at bit 8), the coefficients (2 bits each).
+// Teams of several lanes take CHUNK reactions at a time: each lane leaves its reactions' net rates,
+// rate constants and d q/dT in shared memory, then the team gathers them by species and by
+// Jacobian entry.  What few reactions have (third-body parts, sides of third order) and a single
+// lane's sums are added in place.
 template <bool WJ>
 __device__ __forceinline__ void reaction_loop(const Team& tm, const CellScalars& cs, double P,
                                               const double* __restrict__ lnA_ext) {
-  const double T = cs.T, invT = cs.invT, lnT = cs.lnT;
+  const double T = cs.T, invT = cs.invT;
   const double Ctot = P * invT * INV_R_U;    // sum_k C_k = P / (R T)
-  const double rtp = R_OVER_PATM * T;       // (P_atm / R T)^-1
-  const double irtp = PATM_OVER_R * invT;
-  for (int r = tm.tl; r < NR; r += TEAM) {
-    const int kind = mk_kind[r];
-    const double lA = lnA_ext ? lnA_ext[mk_rorig[r]] : mk_lnA[r];
-    const double kinf = exp(lA + mk_b[r] * lnT - mk_th[r] * invT);
-    double kf = kinf;
-    double dlkf_dT = 0.0, dlkf_dM = 0.0;
+#if TEAM == 1
+#pragma unroll 1
+  for (int r = 0; r < NR; ++r) {
+#else
+#pragma unroll 1
+  for (int ch = 0; ch < NCHUNK; ++ch) {
+    const uint4 run = mk_oseg[mk_osegoff[ch] + tm.tl];
+    double dqT[(CHUNK + TEAM - 1) / TEAM];
+#pragma unroll
+    for (int rd = 0; rd < (CHUNK + TEAM - 1) / TEAM; ++rd) {
+      const int j = rd * TEAM + tm.tl, r = ch * CHUNK + j;
+      if (j < CHUNK && r < NR) {
+#endif
+    // everything the reaction needs from the tables first: they come from L2 mostly
+    const int4 rec = mk_rec[r];
+    const longlong2 kf1 = mk_kfx[r][0], kf2 = mk_kfx[r][1];
+    const int fl = rec.w, kind = (fl >> 4) & 3, dnu = ((fl >> 8) & 31) - 16;
+    // species and coefficient (0: none) of slot i: reactants 0..2, products 3..5
+    auto sp = [&](int i) -> int {
+      const unsigned x = i < 2 ? rec.x : (i < 4 ? rec.y : rec.z);
+      return (i & 1) ? x >> 16 : x & 0xffff;
+    };
+    auto nu = [&](int i) -> int { return (fl >> (13 + 2 * i)) & 3; };
+    const double* lAe = lnA_ext ? &lnA_ext[mk_rorig[r]] : nullptr;
+    const int eff0 = (int)kf2.y, eff1 = (int)(kf2.y >> 32);
     double M = 0.0;
-    if (WJ) dlkf_dT = (mk_b[r] + mk_th[r] * invT) * invT;
     if (kind != ELEM) {
       M = Ctot;
-      for (int e = mk_effoff[r]; e < mk_effoff[r + 1]; ++e) M += mk_effval[e] * tm.at(OFF_C, mk_effsp[e]);
+#pragma unroll 1
+      for (int e = eff0; e < eff1; ++e) M += mk_effval[e] * tm.at(OFF_C, mk_effsp[e]);
     }
-    if (kind >= LIND) {
-      const double k0 = exp(mk_lnA0[r] + mk_b0[r] * lnT - mk_th0[r] * invT);
-      double Pr = k0 * M / kinf;
-      bool floored = false;
-      if (Pr < 1e-300) { Pr = 1e-300; floored = true; }
-      double F = 1.0, dlF_dlPr = 0.0, dlF_dT = 0.0;
-      if (kind == TROE) {
-        const double a = mk_troe[r][0];
-        const double e3 = exp(-T * mk_troe[r][1]);
-        const double e1 = exp(-T * mk_troe[r][2]);
-        const double T2 = mk_troe[r][3];
-        const double e2 = T2 > 0.0 ? exp(-T2 * invT) : 0.0;
-        const double Fc = (1.0 - a) * e3 + a * e1 + e2;
-        const double lFc = log10(Fc);
-        const double c = -0.4 - 0.67 * lFc;
-        const double n = 0.75 - 1.27 * lFc;
-        const double x = log10(Pr) + c;
-        const double d = n - 0.14 * x;
-        const double id = 1.0 / d;
-        const double f1 = x * id;
-        const double den = 1.0 / (1.0 + f1 * f1);
-        const double lF = lFc * den;
-        F = exp(lF * LN10);
+    // log2 K_c = sum_k nu_k log2 exp(s/R - h/RT) + dnu log2(P_atm / R T)
+    Rate q;
+    bool ok = false;
+    if (cs.fx) {
+      fx_i64 lKc = dnu * (FX_LOG2_PATM_R - (cs.l2Tq >> 7));
+#pragma unroll
+      for (int i = 0; i < 6; ++i)
+        if (nu(i)) lKc += (i < 3 ? -nu(i) : nu(i)) * (fx_i64)fx_bits(tm.at(OFF_G, sp(i)));
+      ok = rate_fx<WJ>(r, kind, cs, kf1, kf2.x, lAe, M, lKc, &q);
+    }
+    if (!ok) {
+      double lKc = dnu * (LOG2_PATM_R - cs.l2T);
+#pragma unroll 1
+      for (int i = 0; i < 6; ++i)
+        if (nu(i)) {
+          const double g = tm.at(OFF_G, sp(i));
+          lKc += (i < 3 ? -nu(i) : nu(i)) * (cs.fx ? fx_to_double((fx_i64)fx_bits(g), 52) : g);
+        }
+      Rate qs;  // (its address is taken: kept apart from the registers of the normal path)
+      rate_fp<WJ>(r, kind, T, invT, cs.l2T, lAe ? *lAe : mk_lnA[r], M, lKc, &qs);
+      q = qs;
+    }
+    double fwd = q.kf, rev = q.kr;
+    double dlKc = 0.0;  // T d ln K_c/dT = sum nu'' h/RT - sum nu' h/RT - dnu
+    if (WJ) dlKc = -mk_dnuf[r];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const int n = nu(i);
+      if (n) {
+        const int k = sp(i);
+        const double c = tm.at(OFF_C, k);
+        double& x = i < 3 ? fwd : rev;
+        x *= c;
         if (WJ) {
-          const double g2 = 2.0 * lFc * f1 * den * den;  // -d log10F / d f1
-          if (!floored) dlF_dlPr = -g2 * n * id * id;
-          const double dFc = -(1.0 - a) * mk_troe[r][1] * e3 - a * mk_troe[r][2] * e1 +
-                             (T2 > 0.0 ? T2 * invT * invT * e2 : 0.0);
-          const double df1_dlFc = (-0.67 * n + 1.27 * x) * id * id;
-          const double dlog10F_dlFc = den - g2 * df1_dlFc;
-          dlF_dT = dlog10F_dlFc * dFc / Fc;
+          const double h = tm.at(OFF_HRT, k);
+          dlKc += i < 3 ? dneg(h) : h;
         }
-      }
-      kf = kinf * (Pr / (1.0 + Pr)) * F;
-      if (WJ) {
-        const double g = floored ? 0.0 : 1.0 / (1.0 + Pr) + dlF_dlPr;
-        const double dlk0 = (mk_b0[r] + mk_th0[r] * invT) * invT;
-        dlkf_dM = g / M;
-        dlkf_dT = dlkf_dT + g * (dlk0 - dlkf_dT) + dlF_dT;
-      }
-    }
-    // reverse constant: k_r = k_f / K_c with K_c = prod exp(s/R - h/RT)^nu (P_atm/RT)^dnu
-    double kr = kf;
-    double fwd = kf;
-    const int nre = mk_nre[r], npr = mk_npr[r];
-    for (int i = 0; i < nre; ++i) {
-      const int sp = mk_rsp[r][i];
-      const double c = tm.at(OFF_C, sp), ex = tm.at(OFF_EX, sp);
-      for (int v = 0; v < mk_rnu[r][i]; ++v) { fwd *= c; kr *= ex; }
-    }
-    double rev = 1.0;
-    for (int i = 0; i < npr; ++i) {
-      const int sp = mk_psp[r][i];
-      const double c = tm.at(OFF_C, sp), iex = tm.at(OFF_IEX, sp);
-      for (int v = 0; v < mk_pnu[r][i]; ++v) { rev *= c; kr *= iex; }
-    }
-    const int dnu = mk_dnu[r];
-    for (int v = 0; v < dnu; ++v) kr *= rtp;
-    for (int v = 0; v < -dnu; ++v) kr *= irtp;
-    rev *= kr;
-    const double m = kind == THIRD ? M : 1.0;
-    const double qnet = fwd - rev;
-    const double q = m * qnet;
-    // shared-memory reductions without a return value do not stall the lane (TEAM > 1)
-    for (int i = 0; i < nre; ++i)
-      scatter_add<double>(&tm.at(OFF_OM, mk_rsp[r][i]), nu_times(-mk_rnu[r][i], -mk_rnuf[r][i], q));
-    for (int i = 0; i < npr; ++i)
-      scatter_add<double>(&tm.at(OFF_OM, mk_psp[r][i]), nu_times(mk_pnu[r][i], mk_pnuf[r][i], q));
-    if (WJ) {
-      // d ln Kc / dT = (sum nu'' h/RT - sum nu' h/RT - dnu) / T
-      double dlKc = -mk_dnuf[r];
-      for (int i = 0; i < npr; ++i) dlKc += mk_pnuf[r][i] * tm.at(OFF_HRT, mk_psp[r][i]);
-      for (int i = 0; i < nre; ++i) dlKc -= mk_rnuf[r][i] * tm.at(OFF_HRT, mk_rsp[r][i]);
-      dlKc *= invT;
-      const double dqdT = m * (fwd * dlkf_dT - rev * (dlkf_dT - dlKc));
-      // dq/d[M]: the [M] factor of THIRD reactions, the falloff blend of LIND/TROE
-      const double beta = kind == THIRD ? qnet : (kind == ELEM ? 0.0 : qnet * dlkf_dM);
-      // dq/dC_j of the mass-action products
-      double dq[2 * MAXP];
-      int dsp[2 * MAXP];
-      int nd = 0;
-      for (int i = 0; i < nre; ++i) {
-        const int nu = mk_rnu[r][i];
-        double p = m * kf * mk_rnuf[r][i];
-        for (int i2 = 0; i2 < nre; ++i2) {
-          const double c = tm.at(OFF_C, mk_rsp[r][i2]);
-          const int e = i2 == i ? nu - 1 : mk_rnu[r][i2];
-          for (int v = 0; v < e; ++v) p *= c;
-        }
-        dq[nd] = p;
-        dsp[nd++] = mk_rsp[r][i];
-      }
-      for (int i = 0; i < npr; ++i) {
-        const int nu = mk_pnu[r][i];
-        double p = -m * kr * mk_pnuf[r][i];
-        for (int i2 = 0; i2 < npr; ++i2) {
-          const double c = tm.at(OFF_C, mk_psp[r][i2]);
-          const int e = i2 == i ? nu - 1 : mk_pnu[r][i2];
-          for (int v = 0; v < e; ++v) p *= c;
-        }
-        dq[nd] = p;
-        dsp[nd++] = mk_psp[r][i];
-      }
-      for (int side = 0; side < 2; ++side) {
-        const int np = side == 0 ? nre : npr;
-        for (int i = 0; i < np; ++i) {
-          const int k = side == 0 ? mk_rsp[r][i] : mk_psp[r][i];
-          const int nui = side == 0 ? -mk_rnu[r][i] : mk_pnu[r][i];
-          const double nuk = side == 0 ? -mk_rnuf[r][i] : mk_pnuf[r][i];
-          const int row = smap(k);
-          for (int d = 0; d < nd; ++d) scatter_add<double>(&tm.A(row, smap(dsp[d])), nu_times(nui, nuk, dq[d]));
-          scatter_add<double>(&tm.at(OFF_DOMT, k), nu_times(nui, nuk, dqdT));
-          if (kind != ELEM) {
-            const double nb = nu_times(nui, nuk, beta);
-            scatter_add<double>(&tm.at(OFF_BK, k), nb);
-            for (int e = mk_effoff[r]; e < mk_effoff[r + 1]; ++e)
-              scatter_add<double>(&tm.A(row, smap(mk_effsp[e])), nb * mk_effval[e]);
+        if (n > 1) {
+#pragma unroll 1
+          for (int v = 1; v < n; ++v) {
+            x *= c;
+            if (WJ) {
+              const double h = tm.at(OFF_HRT, k);
+              dlKc += i < 3 ? dneg(h) : h;
+            }
           }
         }
       }
     }
+    const double qnet = fwd - rev;
+    const double qr = kind == THIRD ? M * qnet : qnet;
+#if TEAM == 1
+#pragma unroll 1
+    for (int i = 0; i < 6; ++i)
+      if (nu(i)) tm.at(OFF_OM, sp(i)) += nu_times(i < 3 ? -nu(i) : nu(i), qr);
+#else
+    tm.at(OFF_Q, j) = qr;
+#endif
+    if (WJ) {
+      double dqdT = qnet * q.dlT + rev * (dlKc * invT);
+      if (kind == THIRD) {
+        dqdT *= M;
+        q.kf *= M;
+        q.kr *= M;
+      }
+#if TEAM > 1
+      dqT[rd] = dqdT;
+      tm.at(OFF_KF, j) = q.kf;
+      tm.at(OFF_KF, CHUNK + j) = q.kr;
+#endif
+      if (kind != ELEM) {
+        // dq/d[M]: the [M] factor of THIRD reactions, the falloff blend of LIND/TROE
+        const double beta = kind == THIRD ? qnet : qnet * q.dlM;
+#pragma unroll 1
+        for (int i = 0; i < 6; ++i)
+          if (nu(i)) {
+            const double nb = nu_times(i < 3 ? -nu(i) : nu(i), beta);
+            scatter_add<double>(&tm.at(OFF_BK, sp(i)), nb);
+#pragma unroll 1
+            for (int e = eff0; e < eff1; ++e)
+              scatter_add<double>(&tm.A(smap(sp(i)), smap(mk_effsp[e])), nb * mk_effval[e]);
+          }
+      }
+#if TEAM == 1 || !GATHER_J || HAS_GENERAL
+      if (TEAM == 1 || !GATHER_J || (fl & 0x80)) {
+        // dq/dC_d of the mass-action products, into the rows of every species of the reaction
+#pragma unroll 1
+        for (int d = 0; d < 6; ++d)
+          if (nu(d)) {
+            double p = nu_times(d < 3 ? nu(d) : -nu(d), d < 3 ? q.kf : q.kr);
+#pragma unroll 1
+            for (int i2 = d < 3 ? 0 : 3; i2 < (d < 3 ? 3 : 6); ++i2) {
+              const int e = i2 == d ? nu(d) - 1 : nu(i2);
+#pragma unroll 1
+              for (int v = 0; v < e; ++v) p *= tm.at(OFF_C, sp(i2));
+            }
+#pragma unroll 1
+            for (int i = 0; i < 6; ++i)
+              if (nu(i)) scatter_add<double>(&tm.A(smap(sp(i)), smap(sp(d))), nu_times(i < 3 ? -nu(i) : nu(i), p));
+          }
+      }
+#endif
+#if TEAM == 1
+#pragma unroll 1
+      for (int i = 0; i < 6; ++i)
+        if (nu(i)) tm.at(OFF_DOMT, sp(i)) += nu_times(i < 3 ? -nu(i) : nu(i), dqdT);
+#endif
+    }
+#if TEAM > 1
+      }
+    }
+    tsync();
+    gather_species(tm, ch, run, OFF_OM);
+    if (WJ) {
+#if GATHER_J
+      gather_jacobian(tm, ch);
+#endif
+      tsync();
+#pragma unroll
+      for (int rd = 0; rd < (CHUNK + TEAM - 1) / TEAM; ++rd)
+        if (rd * TEAM + tm.tl < CHUNK) tm.at(OFF_Q, rd * TEAM + tm.tl) = dqT[rd];
+      tsync();
+      gather_species(tm, ch, run, OFF_DOMT);
+    }
+    tsync();
+#endif
   }
+#if TEAM == 1
   tsync();
+#endif
 }
 
 // f from omega: f[0] = dT/dt = -T sum_k (h_k/RT) V omega_k / sum_k n_k cp_k/R,
@@ -512,7 +873,7 @@ __device__ __forceinline__ double source_from_omega(const Team& tm, const CellSc
     if (k < NS - 1) tm.at(of, 1 + k) = cs.V * om;
   }
   hs = team_sum(tm, hs);
-  const double fT = -cs.T * cs.V * hs / cs.cpm;
+  const double fT = -cs.T * cs.V * hs * fx_rcp(cs.cpm);
   if (tm.tl == 0) tm.at(of, 0) = fT;
   tsync();
   return fT;
@@ -529,7 +890,8 @@ __device__ __forceinline__ void zero_rates(const Team& tm, bool with_j) {
 }
 
 // f(y) into slot `of` for the state at slot `oy`.
-__device__ void eval_f(const Team& tm, int oy, int of, double P, const double* lnA_ext) {
+OUTLINE void eval_f(int oy, int of, double P, const double* lnA_ext) {
+  const Team tm = make_team();
   CellScalars cs;
   thermo_conc<false>(tm, oy, P, cs);
   zero_rates(tm, false);
@@ -537,10 +899,11 @@ __device__ void eval_f(const Team& tm, int oy, int of, double P, const double* l
   source_from_omega(tm, cs, of);
 }
 
-// f(y) into `of` and the state Jacobian into A: A = sgn * J + shift * I.
-// sgn = +1, shift = 0 gives J; sgn = -1, shift = 1/(gamma h) gives M = I/(gamma h) - J.
-__device__ void eval_f_jac(const Team& tm, int oy, int of, double P, const double* lnA_ext,
-                           double sgn, double shift) {
+// f(y) into `of` and the state Jacobian into A: J for SGN = 1 (shift = 0), and M = I shift - J with
+// shift = 1/(gamma h) for SGN = -1.
+template <int SGN>
+OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double shift) {
+  const Team tm = make_team();
   CellScalars cs;
   thermo_conc<true>(tm, oy, P, cs);
   zero_rates(tm, true);
@@ -548,54 +911,59 @@ __device__ void eval_f_jac(const Team& tm, int oy, int of, double P, const doubl
   const double fT = source_from_omega(tm, cs, of);
   const double T = cs.T, V = cs.V, invT = cs.invT;
   const double Ctot = P * invT * INV_R_U;
-  const double RTP = 1.0 / Ctot;  // R T / P
+  const double RTP = R_U * T * fx_rcp(P);  // R T / P
   // per species row k (B_k = default-efficiency third-body part, added to every column):
   //   D_k = omega_k - sum_m (d omega_k/dC_m) C_m,
   //   d f_k/d n_j = d omega_k/dC_j - w_j d omega_k/dC_bath + (RT/P)(1 - w_j) D_k
   //               = A_kj + P1_k - w_j P2_k with P1 = B_k + (RT/P) D_k, P2 = A_kb + B_k + (RT/P) D_k,
   //   d f_k / dT = V (D_k / T + d omega_k/dT).
-  for (int k = tm.tl; k < NS; k += TEAM) {
+  // RSPLIT lanes share a row's dot product (and a column's below): the dependent FMAs of a lane set
+  // the time of these passes
+  for (int kk = tm.tl / RSPLIT; kk < NS_PAD; kk += TEAM / RSPLIT) {
+    const int k = kk < NS ? kk : NS - 1;
     const int row = smap(k);
-    // four partial sums: independent FMA chains instead of one NS-long dependent chain
-    double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
-    int j = 0;
-    for (; j + 3 < NS; j += 4) {
+    double d0 = 0.0, d1 = 0.0;
+    int j = tm.tl % RSPLIT;
+    for (; j + RSPLIT < NS; j += 2 * RSPLIT) {
       d0 += tm.A(row, smap(j)) * tm.at(OFF_C, j);
-      d1 += tm.A(row, smap(j + 1)) * tm.at(OFF_C, j + 1);
-      d2 += tm.A(row, smap(j + 2)) * tm.at(OFF_C, j + 2);
-      d3 += tm.A(row, smap(j + 3)) * tm.at(OFF_C, j + 3);
+      d1 += tm.A(row, smap(j + RSPLIT)) * tm.at(OFF_C, j + RSPLIT);
     }
-    for (; j < NS; ++j) d0 += tm.A(row, smap(j)) * tm.at(OFF_C, j);
-    const double dot = (d0 + d1) + (d2 + d3);
-    const double Bk = tm.at(OFF_BK, k);
-    const double D = tm.at(OFF_OM, k) - dot - Bk * Ctot;
-    tm.at(OFF_AL, k) = tm.A(row, 0) + Bk + RTP * D;
-    tm.at(OFF_BE, k) = Bk + RTP * D;
-    tm.at(OFF_JT, k) = V * (D * invT + tm.at(OFF_DOMT, k));
+    if (j < NS) d0 += tm.A(row, smap(j)) * tm.at(OFF_C, j);
+    const double dot = rsplit_sum(d0 + d1);
+    if (kk < NS && tm.tl % RSPLIT == 0) {
+      const double Bk = tm.at(OFF_BK, k);
+      const double D = tm.at(OFF_OM, k) - dot - Bk * Ctot;
+      const double be = Bk + RTP * D;
+      tm.at(OFF_AL, k) = tm.A(row, 0) + be;
+      tm.at(OFF_BE, k) = be;
+      tm.at(OFF_JT, k) = V * (D * invT + tm.at(OFF_DOMT, k));
+    }
   }
   tsync();
-  // species rows, w_j = W_j / W_bath
+  // species rows, w_j = W_j / W_bath (the diagonal shift of M comes last)
 #if TEAM == 1
   for (int i = 1; i < NEQ; ++i) {
-    const int k = i - 1;
-    const double al = tm.at(OFF_AL, k), be = tm.at(OFF_BE, k);
+    const double al = tm.at(OFF_AL, i - 1), be = tm.at(OFF_BE, i - 1);
     for (int l = 1; l < NEQ; ++l) {
       const double w = mk_wratio[l - 1];
-      const double J = tm.A(i, l) - w * al + be;
-      tm.A(i, l) = sgn * J + (i == l ? shift : 0.0);
+      tm.A(i, l) = SGN > 0 ? (tm.A(i, l) + be) - w * al : w * al - (tm.A(i, l) + be);
     }
-    tm.A(i, 0) = sgn * tm.at(OFF_JT, k);
+    tm.A(i, 0) = SGN > 0 ? tm.at(OFF_JT, i - 1) : dneg(tm.at(OFF_JT, i - 1));
   }
 #else
-  for (int e = tm.tl; e < (NEQ - 1) * NEQ; e += TEAM) {
-    const int i = 1 + e / NEQ, l = e - (i - 1) * NEQ;
-    const int k = i - 1;
-    if (l == 0) {
-      tm.A(i, 0) = sgn * tm.at(OFF_JT, k);
-    } else {
-      const double w = mk_wratio[l - 1];
-      const double J = tm.A(i, l) - w * tm.at(OFF_AL, k) + tm.at(OFF_BE, k);
-      tm.A(i, l) = sgn * J + (i == l ? shift : 0.0);
+  {
+    int i = 1 + tm.tl / NEQ, l = tm.tl % NEQ;
+    for (int e = tm.tl; e < (NEQ - 1) * NEQ; e += TEAM) {
+      const int k = i - 1;
+      if (l == 0) {
+        tm.A(i, 0) = SGN > 0 ? tm.at(OFF_JT, k) : dneg(tm.at(OFF_JT, k));
+      } else {
+        const double w = mk_wratio[l - 1], al = tm.at(OFF_AL, k), a = tm.A(i, l) + tm.at(OFF_BE, k);
+        tm.A(i, l) = SGN > 0 ? a - w * al : w * al - a;
+      }
+      i += TEAM / NEQ;
+      l += TEAM % NEQ;
+      if (l >= NEQ) { l -= NEQ; ++i; }
     }
   }
 #endif
@@ -604,38 +972,42 @@ __device__ void eval_f_jac(const Team& tm, int oy, int of, double P, const doubl
   // V omega_k, bath included); dQ/dn_j = T sum_k (h_k/RT) J_kj, dQ/dT = sum_k cp_k f'_k +
   // T sum_k (h_k/RT) J_kT; d cpm/dn_j = cp_j - w_j cp_bath, d cpm/dT = sum_k n_k dcp_k/dT.
   const double hb = tm.at(OFF_HRT, BATH), alb = tm.at(OFF_AL, BATH), beb = tm.at(OFF_BE, BATH);
-  const double icpm = 1.0 / cs.cpm;
+  const double icpm = fx_rcp(cs.cpm);
   double cpf = 0.0;  // sum_k cp_k omega_k, a team reduction rather than one lane's loop
   for (int k = tm.tl; k < NS; k += TEAM) cpf += tm.at(OFF_CP, k) * tm.at(OFF_OM, k);
   cpf = team_sum(tm, cpf);
-  for (int l = tm.tl; l < NEQ; l += TEAM) {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    int i = 1;
-    for (; i + 3 < NEQ; i += 4) {
+  for (int ll = tm.tl / RSPLIT; ll < NS_PAD; ll += TEAM / RSPLIT) {
+    const int l = ll < NEQ ? ll : NEQ - 1;
+    double s0 = 0.0, s1 = 0.0;
+    int i = 1 + tm.tl % RSPLIT;
+    for (; i + RSPLIT < NEQ; i += 2 * RSPLIT) {
       s0 += tm.at(OFF_HRT, i - 1) * tm.A(i, l);
-      s1 += tm.at(OFF_HRT, i) * tm.A(i + 1, l);
-      s2 += tm.at(OFF_HRT, i + 1) * tm.A(i + 2, l);
-      s3 += tm.at(OFF_HRT, i + 2) * tm.A(i + 3, l);
+      s1 += tm.at(OFF_HRT, i - 1 + RSPLIT) * tm.A(i + RSPLIT, l);
     }
-    for (; i < NEQ; ++i) s0 += tm.at(OFF_HRT, i - 1) * tm.A(i, l);
-    double s = (s0 + s1) + (s2 + s3);
-    if (l > 0) s -= tm.at(OFF_HRT, l - 1) * shift;  // remove the diagonal shift of M
-    s *= sgn;  // the rows above carry the sign
-    double val;
-    if (l == 0) {
-      s += hb * tm.at(OFF_JT, BATH);
-      const double dQdT = cpf * V + T * s;
-      val = -(dQdT + fT * cs.dcpm) * icpm;
-    } else {
-      const double w = mk_wratio[l - 1];
-      const double Jb = tm.A(0, l) - w * alb + beb;  // bath row, before it is overwritten
-      s += hb * Jb;
-      const double dcpm = tm.at(OFF_CP, l - 1) - w * tm.at(OFF_CP, BATH);
-      val = -(T * s + fT * dcpm) * icpm;
+    if (i < NEQ) s0 += tm.at(OFF_HRT, i - 1) * tm.A(i, l);
+    double s = rsplit_sum(s0 + s1);
+    if (SGN < 0) s = dneg(s);  // the rows above carry the sign
+    if (ll < NEQ && tm.tl % RSPLIT == 0) {
+      double val;
+      if (l == 0) {
+        s += hb * tm.at(OFF_JT, BATH);
+        const double dQdT = cpf * V + T * s;
+        val = -(dQdT + fT * cs.dcpm) * icpm;
+      } else {
+        const double w = mk_wratio[l - 1];
+        const double Jb = tm.A(0, l) - w * alb + beb;  // bath row, before it is overwritten
+        s += hb * Jb;
+        const double dcpm = tm.at(OFF_CP, l - 1) - w * tm.at(OFF_CP, BATH);
+        val = -(T * s + fT * dcpm) * icpm;
+      }
+      tm.A(0, l) = SGN > 0 ? val : dneg(val);
     }
-    tm.A(0, l) = sgn * val + (l == 0 ? shift : 0.0);
   }
   tsync();
+  if (SGN < 0) {
+    for (int i = tm.tl; i < NEQ; i += TEAM) tm.A(i, i) += shift;
+    tsync();
+  }
 }
 
 // ------------------------------------------------------------------------------ LU + solves
@@ -670,7 +1042,7 @@ __device__ __forceinline__ void lu_panel(const Team& tm, int c) {
     p = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (unsigned)p : 0xffffffffu);
   }
   __syncwarp();  // the updated column is visible to the whole warp
-  const double inv = 1.0 / tm.A(p, c);
+  const double inv = fx_rcp(tm.A(p, c));
   if (tm.tl == 0) {
     tm.base[LU_INV] = inv;
     reinterpret_cast<int*>(&tm.base[LU_PIV])[0] = p;
@@ -684,7 +1056,8 @@ __device__ __forceinline__ void lu_panel(const Team& tm, int c) {
 // In-place LU with partial pivoting of A (N x N): largest |a| in the column, lowest row on
 // ties.  1/U_kk replaces U_kk on the diagonal, the composed row permutation (row i of P A is row
 // perm[i] of A) goes to OFF_PERM, and the single-lane layout also keeps the pivot sequence.
-__device__ void lu_factor(const Team& tm) {
+OUTLINE void lu_factor() {
+  const Team tm = make_team();
 #if TEAM == 1
   for (int k = 0; k < NEQ; ++k) {
     int p = k;
@@ -696,7 +1069,7 @@ __device__ void lu_factor(const Team& tm) {
     tm.piv(k) = p;
     if (p != k)
       for (int j = 0; j < NEQ; ++j) { const double t = tm.A(k, j); tm.A(k, j) = tm.A(p, j); tm.A(p, j) = t; }
-    const double inv = 1.0 / tm.A(k, k);
+    const double inv = fx_rcp(tm.A(k, k));
     tm.invd(k) = inv;
     for (int i = k + 1; i < NEQ; ++i) {
       const double l = tm.A(i, k) * inv;
@@ -808,7 +1181,7 @@ __device__ void lu_factor(const Team& tm) {
     // 1/pivot and the column scale by the first warp only: a warp-level FP64 instruction costs the
     // same pipe time whatever its lane count, so the other warps must not repeat the division
     if (tm.tl < 32) {
-      const double inv = 1.0 / tm.A(k, k);
+      const double inv = fx_rcp(tm.A(k, k));
       __syncwarp(msk);  // every lane has read U_kk before lane 0 replaces it by its inverse
       if (tm.tl == 0) {
         tm.invd(k) = inv;
@@ -843,7 +1216,8 @@ __device__ __forceinline__ void solve_bar() {
 
 // Solve (LU) x = b in place on the vector at slot ob.  With TEAM > 1 only the first warp works,
 // except for teams of four or more warps, where warp w holds rows 32w..32w+31.
-__device__ void lu_solve(const Team& tm, int ob) {
+OUTLINE void lu_solve(int ob) {
+  const Team tm = make_team();
 #if TEAM == 1
   for (int k = 0; k < NEQ; ++k) {
     const int p = tm.piv(k);
@@ -983,7 +1357,8 @@ __device__ void lu_solve(const Team& tm, int ob) {
 #if TEAM > 1
 // Column-oriented solve by the team's first warp through shared memory (the adjoint kernels use it: it needs
 // no registers for the vector, and the adjoint kernels run at their register cap).
-__device__ void lu_solve_col(const Team& tm, int ob) {
+OUTLINE void lu_solve_col(int ob) {
+  const Team tm = make_team();
   if (tm.tl < 32) {
     const int ln = tm.tl & (WL - 1);
     const unsigned msk = team_mask();
@@ -1025,8 +1400,8 @@ __device__ void lu_solve_col(const Team& tm, int ob) {
 // One attempt of the s-stage Rosenbrock method of the generated header (Sec. 2.3, transformed
 // form): coefficients rk_a, rk_c, rk_m, rk_e, gamma RGAM, RS stages; rk_newf[i] says whether stage
 // i needs f at a new argument (1), reuses the previous stage's f (0: equal argument), or uses
-// f(y) (2: the argument is y).  Size hh from y (OFF_Y): y_new into OFF_YT; returns the weighted
-// RMS error (infinity if anything is non-finite).
+// f(y) (2: the argument is y).  Size hh from y (OFF_Y): y_new into OFF_YT; returns the square of
+// the weighted RMS error (infinity if anything is non-finite).
 // REG_SOLVE selects the register-resident stage solves, used for state vectors of more than 64
 // entries (GB300, 111 species: +5% cells/s; at 53 species they measured 12% slower than the
 // column-oriented sweep, at 13 species no different).  The adjoint's replay takes the column-oriented
@@ -1035,11 +1410,11 @@ template <bool REG_SOLVE>
 __device__ __forceinline__ void stage_solve(const Team& tm, int ob) {
 #if TEAM > 1
   if (!REG_SOLVE) {
-    lu_solve_col(tm, ob);
+    lu_solve_col(ob);
     return;
   }
 #endif
-  lu_solve(tm, ob);
+  lu_solve(ob);
 }
 
 template <bool REG_SOLVE = (NB >= 3)>
@@ -1059,7 +1434,7 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
       }
       tsync();
     }
-    eval_f(tm, st == 0 ? OFF_Y : OFF_YT, OFF_F, P, lnA_ext);
+    eval_f(st == 0 ? OFF_Y : OFF_YT, OFF_F, P, lnA_ext);
     const int ou = UOFF(st);
     for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(ou, i) = hh * tm.at(OFF_F, i);
     tsync();
@@ -1069,7 +1444,7 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
   // of I/(gamma h) - W when it was made for this step size and is young enough)
   const bool reuse = wc && wc[WC_H] == hh && wc[WC_AGE] < WAGE_MAX;
   if (reuse) {
-    eval_f(tm, OFF_Y, OFF_U1, P, lnA_ext);
+    eval_f(OFF_Y, OFF_U1, P, lnA_ext);
     for (int e = tm.tl; e < NEQ * NEQ; e += TEAM) tm.at(OFF_A, e) = wc[e];
     for (int e = tm.tl; e < PACKED_INTS(NEQ); e += TEAM) {
       tm.at(OFF_PERM, e) = wc[WC_PERM + e];
@@ -1079,13 +1454,13 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
     }
     tsync();
   } else {
-    eval_f_jac(tm, OFF_Y, OFF_U1, P, lnA_ext, -1.0, 1.0 / (RGAM * hh));
+    eval_f_jac<-1>(OFF_Y, OFF_U1, P, lnA_ext, fx_rcp(RGAM * hh));
   }
   if (rho && !reuse) {
     // stiffness estimate: Gershgorin bound of the Jacobian scaled by the error weights,
     // max_i sum_j |J_ij| w_j / w_i with w = atol + rtol |y| (J_ij = -A_ij off the diagonal,
     // shift - A_ii on it)
-    const double shift = 1.0 / (RGAM * hh);
+    const double shift = fx_rcp(RGAM * hh);
     double mx = 0.0;
     for (int i = tm.tl; i < NEQ; i += TEAM) {
       double sum = 0.0;
@@ -1103,7 +1478,7 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
   tsync();
 #endif
   if (!reuse) {
-    lu_factor(tm);
+    lu_factor();
     if (wc) {  // keep the factorisation for later attempts of this size
       for (int e = tm.tl; e < NEQ * NEQ; e += TEAM) wc[e] = tm.at(OFF_A, e);
       for (int e = tm.tl; e < PACKED_INTS(NEQ); e += TEAM) {
@@ -1116,7 +1491,7 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
     }
   }
   stage_solve<REG_SOLVE>(tm, OFF_U1);
-  const double ih = 1.0 / hh;
+  const double ih = fx_rcp(hh);
 #pragma unroll
   for (int st = 1; st < RS; ++st) {
     if (rk_newf[st] == 1) {
@@ -1127,7 +1502,7 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
         tm.at(OFF_YT, i) = v;
       }
       tsync();
-      eval_f(tm, OFF_YT, OFF_F, P, lnA_ext);
+      eval_f(OFF_YT, OFF_F, P, lnA_ext);
     }
 #if NEED_F0
     const int of = rk_newf[st] == 2 ? OFF_F0 : OFF_F;
@@ -1136,10 +1511,10 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
 #endif
     const int ou = UOFF(st);
     for (int i = tm.tl; i < NEQ; i += TEAM) {
-      double v = tm.at(of, i);
+      double v = 0.0;
       for (int j = 0; j < st; ++j)
-        if (rk_c[st * RS + j] != 0.0) v += (rk_c[st * RS + j] * ih) * tm.at(UOFF(j), i);
-      tm.at(ou, i) = v;
+        if (rk_c[st * RS + j] != 0.0) v += rk_c[st * RS + j] * tm.at(UOFF(j), i);
+      tm.at(ou, i) = fma(ih, v, tm.at(of, i));
     }
     tsync();
     stage_solve<REG_SOLVE>(tm, ou);
@@ -1160,15 +1535,15 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
     tm.at(OFF_YT, i) = yn;
     const double ay = fabs(y), an = fabs(yn);
     const double sc = atol + rtol * (ay > an ? ay : an);
-    const double z = e / sc;
+    const double z = e * fx_rcp(sc);
     acc += z * z;
     if (!isfinite(yn)) bad = true;
   }
   acc = team_sum(tm, acc);
   bad = team_any(tm, bad);
   tsync();
-  const double err = sqrt(acc / NEQ);
-  return (bad || !isfinite(err)) ? __longlong_as_double(0x7ff0000000000000LL) : err;
+  const double err2 = acc * (1.0 / NEQ);
+  return (bad || !isfinite(err2)) ? __longlong_as_double(0x7ff0000000000000LL) : err2;
 }
 
 // Controller state of one cell (team-uniform: every lane holds the same values).
@@ -1196,23 +1571,19 @@ __device__ __forceinline__ void ros4_advance(const Team& tm, Ctl& c, double P, d
   if (c.h < h_min) { c.status = ST_H_UNDERFLOW; c.done = true; return; }
   const bool last = c.t + 1.0001 * c.h >= dt;
   const double hh = last ? dt - c.t : c.h;
-  const double err = ros4_attempt(tm, P, hh, rtol, atol, lnA_ext,
+  const double err2 = ros4_attempt(tm, P, hh, rtol, atol, lnA_ext,
                                   (c.want_rho && c.attempts == 0) ? &c.rho : nullptr, c.wc);
   c.attempts++;
-  const bool finite = isfinite(err);
+  const bool finite = isfinite(err2);
   double fac = 0.2;
   if (finite) {
-    const double e = err > 1e-10 ? err : 1e-10;
-#if RORDER == 4
-    fac = 0.9 / sqrt(sqrt(e));  // 0.9 err^(-1/order)
-#elif RORDER == 3
-    fac = 0.9 / cbrt(e);
-#else
-    fac = 0.9 * pow(e, -1.0 / RORDER);
-#endif
+    // 0.9 err^(-1/order), every lane on the integer pipe (two square roots and a division would take
+    // about 1,300 clocks of FP64 latency)
+    const double e = err2 > 1e-20 ? err2 : 1e-20;
+    fac = 0.9 * fx_exp2(-fx_log2(e) / (2 * RORDER));
     fac = fac < 0.2 ? 0.2 : (fac > 6.0 ? 6.0 : fac);
   }
-  if (finite && err <= 1.0) {
+  if (finite && err2 <= 1.0) {
     for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(OFF_Y, i) = tm.at(OFF_YT, i);
     if (c.wc && tm.tl == 0) c.wc[WC_AGE] += 1.0;  // the cached factorisation ages per accepted step
     tsync();
@@ -1236,21 +1607,6 @@ __device__ __forceinline__ void ros4_advance(const Team& tm, Ctl& c, double P, d
 }
 
 // ------------------------------------------------------------------------------ cell I/O
-
-__device__ __forceinline__ Team make_team(double* smem) {
-  Team tm;
-#if TEAM == 1
-  tm.base = smem + threadIdx.x;
-  tm.tl = 0;
-#elif TEAM <= 32
-  tm.base = smem + (threadIdx.x / TEAM) * TSTRIDE;
-  tm.tl = threadIdx.x & (TEAM - 1);
-#else
-  tm.base = smem;
-  tm.tl = threadIdx.x;
-#endif
-  return tm;
-}
 
 // y = [T, Y_k / W_k] into OFF_Y; returns false if any input is non-finite
 __device__ __forceinline__ bool load_cell(const Team& tm, long long c, const double* T, const double* Y,
@@ -1308,15 +1664,14 @@ extern "C" __global__ void __launch_bounds__(TPB)
 chem_eval_source_k(long long n_cells, const double* __restrict__ T, const double* __restrict__ P,
                    const double* __restrict__ n, double* __restrict__ f, long long ld,
                    const double* __restrict__ lnA_ext) {
-  extern __shared__ double smem[];
-  const Team tm = make_team(smem);
+  const Team tm = make_team();
   const long long team_id = (long long)blockIdx.x * NTEAM + (TEAM <= 32 ? threadIdx.x / TEAM : 0);
   const long long stride = (long long)gridDim.x * NTEAM;
   for (long long c = team_id; c < n_cells; c += stride) {
     if (tm.tl == 0) tm.at(OFF_Y, 0) = T[c];
     for (int k = tm.tl; k < NS - 1; k += TEAM) tm.at(OFF_Y, 1 + k) = n[k * ld + c];
     tsync();
-    eval_f(tm, OFF_Y, OFF_F, P[c], lnA_ext);
+    eval_f(OFF_Y, OFF_F, P[c], lnA_ext);
     for (int i = tm.tl; i < NEQ; i += TEAM) f[i * ld + c] = tm.at(OFF_F, i);
     tsync();
   }
@@ -1326,15 +1681,14 @@ extern "C" __global__ void __launch_bounds__(TPB)
 chem_eval_jacobian_k(long long n_cells, const double* __restrict__ T, const double* __restrict__ P,
                      const double* __restrict__ n, double* __restrict__ J, long long ld,
                      const double* __restrict__ lnA_ext) {
-  extern __shared__ double smem[];
-  const Team tm = make_team(smem);
+  const Team tm = make_team();
   const long long team_id = (long long)blockIdx.x * NTEAM + (TEAM <= 32 ? threadIdx.x / TEAM : 0);
   const long long stride = (long long)gridDim.x * NTEAM;
   for (long long c = team_id; c < n_cells; c += stride) {
     if (tm.tl == 0) tm.at(OFF_Y, 0) = T[c];
     for (int k = tm.tl; k < NS - 1; k += TEAM) tm.at(OFF_Y, 1 + k) = n[k * ld + c];
     tsync();
-    eval_f_jac(tm, OFF_Y, OFF_U1, P[c], lnA_ext, 1.0, 0.0);  // f goes to U1: F aliases J scratch
+    eval_f_jac<1>(OFF_Y, OFF_U1, P[c], lnA_ext, 0.0);  // f goes to U1: F aliases J scratch
     for (int e = tm.tl; e < NEQ * NEQ; e += TEAM) J[(long long)e * ld + c] = tm.at(OFF_A, e);
     tsync();
   }
@@ -1378,8 +1732,7 @@ chem_integrate_k(long long n_cells, double* __restrict__ T, const double* __rest
                  int tape_cap, int interval, const int* __restrict__ order,
                  const unsigned int* __restrict__ order_count, int keep_failed,
                  int* __restrict__ cell_method, int auto_mode, double* __restrict__ jac_cache) {
-  extern __shared__ double smem[];
-  const Team tm = make_team(smem);
+  const Team tm = make_team();
   long long cell = -1;
   double Pc = 0.0;
   Ctl c;
@@ -1561,8 +1914,7 @@ extern "C" __global__ void __launch_bounds__(TPB)
 chem_plain_init_k(long long n_cells, const double* __restrict__ T, const double* __restrict__ Y,
                   long long ld, double dt, const double* __restrict__ h_in, double T_min,
                   double* wy, double* wt, double* wh, int* wflags, int* watt, int* wst) {
-  extern __shared__ double smem[];
-  const Team tm = make_team(smem);
+  const Team tm = make_team();
   const long long team_id = (long long)blockIdx.x * NTEAM + (TEAM <= 32 ? threadIdx.x / TEAM : 0);
   const long long stride = (long long)gridDim.x * NTEAM;
   for (long long c = team_id; c < n_cells; c += stride) {
@@ -1590,8 +1942,7 @@ chem_plain_attempt_k(long long n_cells, double* __restrict__ T, const double* __
                      int* __restrict__ attempts_out, const double* __restrict__ lnA_ext,
                      int max_steps, double h_min, double* wy, double* wt, double* wh, int* wflags,
                      int* watt, int* wst, unsigned int* active_count) {
-  extern __shared__ double smem[];
-  const Team tm = make_team(smem);
+  const Team tm = make_team();
   const long long team_id = (long long)blockIdx.x * NTEAM + (TEAM <= 32 ? threadIdx.x / TEAM : 0);
   const long long stride = (long long)gridDim.x * NTEAM;
   for (long long cell = team_id; cell < n_cells; cell += stride) {
@@ -1662,8 +2013,9 @@ __device__ __forceinline__ DD operator-(DD a, DD b) { return mk(a.v - b.v, a.d -
 __device__ __forceinline__ DD operator-(DD a) { return mk(-a.v, -a.d); }
 __device__ __forceinline__ DD operator*(DD a, DD b) { return mk(a.v * b.v, a.d * b.v + a.v * b.d); }
 __device__ __forceinline__ DD operator/(DD a, DD b) {
-  const double q = a.v / b.v;
-  return mk(q, (a.d - q * b.d) / b.v);
+  const double rb = fx_rcp(b.v);
+  const double q = a.v * rb;
+  return mk(q, (a.d - q * b.d) * rb);
 }
 __device__ __forceinline__ DD operator+(DD a, double b) { return mk(a.v + b, a.d); }
 __device__ __forceinline__ DD operator+(double b, DD a) { return mk(a.v + b, a.d); }
@@ -1671,14 +2023,23 @@ __device__ __forceinline__ DD operator-(DD a, double b) { return mk(a.v - b, a.d
 __device__ __forceinline__ DD operator-(double b, DD a) { return mk(b - a.v, -a.d); }
 __device__ __forceinline__ DD operator*(DD a, double b) { return mk(a.v * b, a.d * b); }
 __device__ __forceinline__ DD operator*(double b, DD a) { return mk(a.v * b, a.d * b); }
-__device__ __forceinline__ DD operator/(DD a, double b) { return mk(a.v / b, a.d / b); }
+__device__ __forceinline__ DD operator/(DD a, double b) { const double rb = fx_rcp(b); return mk(a.v * rb, a.d * rb); }
 __device__ __forceinline__ DD operator/(double b, DD a) {
-  const double q = b / a.v;
-  return mk(q, -q * a.d / a.v);
+  const double ra = fx_rcp(a.v);
+  const double q = b * ra;
+  return mk(q, -q * a.d * ra);
 }
-__device__ __forceinline__ DD exp(DD a) { const double e = exp(a.v); return mk(e, e * a.d); }
-__device__ __forceinline__ DD log(DD a) { return mk(log(a.v), a.d / a.v); }
-__device__ __forceinline__ DD log10(DD a) { return mk(log10(a.v), a.d / (a.v * LN10)); }
+// value functions on the integer pipe (fx_*)
+__device__ __forceinline__ double xexp(double a) { return fx_exp(a); }
+__device__ __forceinline__ double xlog(double a) { return fx_log(a); }
+__device__ __forceinline__ double xlog10(double a) { return fx_log(a) * (1.0 / LN10); }
+__device__ __forceinline__ double xdiv(double a, double b) { return a * fx_rcp(b); }
+__device__ __forceinline__ DD xexp(DD a) { const double e = fx_exp(a.v); return mk(e, e * a.d); }
+__device__ __forceinline__ DD xlog(DD a) { return mk(fx_log(a.v), a.d * fx_rcp(a.v)); }
+__device__ __forceinline__ DD xlog10(DD a) { return mk(fx_log(a.v) * (1.0 / LN10), a.d * fx_rcp(a.v) * (1.0 / LN10)); }
+__device__ __forceinline__ DD xdiv(DD a, DD b) { return a / b; }
+__device__ __forceinline__ DD xdiv(double a, DD b) { return a / b; }
+__device__ __forceinline__ DD xdiv(DD a, double b) { return a / b; }
 __device__ __forceinline__ double vof(double a) { return a; }
 __device__ __forceinline__ double vof(DD a) { return a.v; }
 __device__ __forceinline__ double dof(double a) { return 0.0; }
@@ -1749,14 +2110,15 @@ __device__ __forceinline__ S team_sum_s(const Team& tm, S v, S* red) {
 // phi(y) = v^T f(y) = sum_k atilde_k omega_k with atilde_k = V v_{1+k} [k < bath]
 // - v_T T V (h_k/RT) / cpm; gy = sum_k atilde_k d omega_k/dy + sum_k omega_k d atilde_k/dy.
 template <class S>
-__device__ void vjp(const Team& tm, double P, const double* __restrict__ lnA_ext) {
+OUTLINE void vjp(double P, const double* __restrict__ lnA_ext) {
+  const Team tm = make_team();
   S* sb = reinterpret_cast<S*>(&tm.base[AOFF_S]);
   S* Y = sb + VS_Y;
   const double* v = &tm.base[AOFF_V];
   double* gp = &tm.base[AOFF_GP];
   const S T = Y[0];
-  const S invT = 1.0 / T;
-  const S lnT = log(T);
+  const S invT = xdiv(1.0, T);
+  const S lnT = xlog(T);
   const S Z = szero<S>();
   S wsum = Z, nsum = Z;
   for (int k = tm.tl; k < NS - 1; k += TEAM) {
@@ -1767,8 +2129,8 @@ __device__ void vjp(const Team& tm, double P, const double* __restrict__ lnA_ext
   wsum = team_sum_s(tm, wsum, red);
   nsum = team_sum_s(tm, nsum, red);
   const S nb = (1.0 - wsum) * mk_invW[BATH];
-  const S V = (nsum + nb) * R_U * T / P;
-  const S invV = 1.0 / V;
+  const S V = (nsum + nb) * R_U * T * fx_rcp(P);
+  const S invV = xdiv(1.0, V);
   S cpm = Z, dcpm = Z;
   for (int k = tm.tl; k < NS; k += TEAM) {
     const S n = k < NS - 1 ? Y[1 + k] : nb;
@@ -1782,11 +2144,11 @@ __device__ void vjp(const Team& tm, double P, const double* __restrict__ lnA_ext
     const S hRT = hh[0] + T * (hh[1] + T * (hh[2] + T * (hh[3] + T * hh[4]))) + hh[5] * invT;
     const S sR = s[0] * lnT + s[6] + T * (s[1] + T * (s[2] + T * (s[3] + T * s[4])));
     const S dcp = d[0] + T * (d[1] + T * (d[2] + T * d[3]));
-    const S ex = exp(sR - hRT);
+    const S ex = xexp(sR - hRT);
     sb[VS_CP + k] = cp;
     sb[VS_HRT + k] = hRT;
     sb[VS_EX + k] = ex;
-    sb[VS_IEX + k] = 1.0 / ex;
+    sb[VS_IEX + k] = xdiv(1.0, ex);
     sb[VS_DCP + k] = dcp;
     sb[VS_CB + k] = Z;
     cpm = cpm + n * cp;
@@ -1795,20 +2157,20 @@ __device__ void vjp(const Team& tm, double P, const double* __restrict__ lnA_ext
   cpm = team_sum_s(tm, cpm, red);
   dcpm = team_sum_s(tm, dcpm, red);
   const double vT = v[0];
-  const S kT = vT * T * V / cpm;
+  const S kT = xdiv(vT * T * V, cpm);
   for (int k = tm.tl; k < NS; k += TEAM) {
     const S a0 = k < NS - 1 ? V * v[1 + k] : Z;
     sb[VS_AT + k] = a0 - kT * sb[VS_HRT + k];
   }
   tsync();
-  const S Ctot = P * invT / R_U;
-  const S rtp = R_U * T / P_ATM;
-  const S irtp = 1.0 / rtp;
+  const S Ctot = P * invT * INV_R_U;
+  const S rtp = R_OVER_PATM * T;
+  const S irtp = PATM_OVER_R * invT;
   S Tbar = Z, Bbar = Z;
   for (int r = tm.tl; r < NR; r += TEAM) {
     const int kind = mk_kind[r];
     const double lA = lnA_ext ? lnA_ext[mk_rorig[r]] : mk_lnA[r];
-    const S kinf = exp(lA + mk_b[r] * lnT - mk_th[r] * invT);
+    const S kinf = xexp(lA + mk_b[r] * lnT - mk_th[r] * invT);
     S kf = kinf;
     S dlkf_dT = (mk_b[r] + mk_th[r] * invT) * invT;
     S dlkf_dM = Z;
@@ -1819,39 +2181,39 @@ __device__ void vjp(const Team& tm, double P, const double* __restrict__ lnA_ext
       for (int e = mk_effoff[r]; e < mk_effoff[r + 1]; ++e) M = M + mk_effval[e] * sb[VS_C + mk_effsp[e]];
     }
     if (kind >= LIND) {
-      const S k0 = exp(mk_lnA0[r] + mk_b0[r] * lnT - mk_th0[r] * invT);
-      S Pr = k0 * M / kinf;
+      const S k0 = xexp(mk_lnA0[r] + mk_b0[r] * lnT - mk_th0[r] * invT);
+      S Pr = xdiv(k0 * M, kinf);
       bool floored = false;
       if (vof(Pr) < 1e-300) { Pr = Z + 1e-300; floored = true; }
       S F = Z + 1.0, dlF_dlPr = Z, dlF_dT = Z;
       if (kind == TROE) {
         const double a = mk_troe[r][0];
-        const S e3 = exp(-T * mk_troe[r][1]);
-        const S e1 = exp(-T * mk_troe[r][2]);
+        const S e3 = xexp(-T * mk_troe[r][1]);
+        const S e1 = xexp(-T * mk_troe[r][2]);
         const double T2 = mk_troe[r][3];
-        const S e2 = T2 > 0.0 ? exp(-T2 * invT) : Z;
+        const S e2 = T2 > 0.0 ? xexp(-T2 * invT) : Z;
         const S Fc = (1.0 - a) * e3 + a * e1 + e2;
-        const S lFc = log10(Fc);
+        const S lFc = xlog10(Fc);
         const S c = -0.4 - 0.67 * lFc;
         const S n = 0.75 - 1.27 * lFc;
-        const S x = log10(Pr) + c;
+        const S x = xlog10(Pr) + c;
         const S d = n - 0.14 * x;
-        const S id = 1.0 / d;
+        const S id = xdiv(1.0, d);
         const S f1 = x * id;
-        const S den = 1.0 / (1.0 + f1 * f1);
+        const S den = xdiv(1.0, 1.0 + f1 * f1);
         const S lF = lFc * den;
-        F = exp(lF * LN10);
+        F = xexp(lF * LN10);
         const S g2 = 2.0 * lFc * f1 * den * den;
         if (!floored) dlF_dlPr = -g2 * n * id * id;
         const S dFc = -(1.0 - a) * mk_troe[r][1] * e3 - a * mk_troe[r][2] * e1 +
                       (T2 > 0.0 ? T2 * invT * invT * e2 : Z);
         const S df1_dlFc = (-0.67 * n + 1.27 * x) * id * id;
-        dlF_dT = (den - g2 * df1_dlFc) * dFc / Fc;
+        dlF_dT = (den - g2 * df1_dlFc) * xdiv(dFc, Fc);
       }
-      kf = kinf * (Pr / (1.0 + Pr)) * F;
-      const S g = floored ? Z : 1.0 / (1.0 + Pr) + dlF_dlPr;
+      kf = kinf * xdiv(Pr, 1.0 + Pr) * F;
+      const S g = floored ? Z : xdiv(1.0, 1.0 + Pr) + dlF_dlPr;
       const S dlk0 = (mk_b0[r] + mk_th0[r] * invT) * invT;
-      dlkf_dM = g / M;
+      dlkf_dM = xdiv(g, M);
       dlkf_dT = dlkf_dT + g * (dlk0 - dlkf_dT) + dlF_dT;
       one_minus_g = 1.0 - g;
     }
@@ -1933,12 +2295,12 @@ __device__ void vjp(const Team& tm, double P, const double* __restrict__ lnA_ext
   vw = team_sum_s(tm, vw, red);
   Dbar = team_sum_s(tm, Dbar, red);
   tsync();
-  const S Sp = vw - vT * T * Q / cpm;  // sum_k omega_k atilde_k / V
-  const S RTP = R_U * T / P;
-  const S icpm2 = 1.0 / (cpm * cpm);
+  const S Sp = vw - xdiv(vT * T * Q, cpm);  // sum_k omega_k atilde_k / V
+  const S RTP = R_U * T * fx_rcp(P);
+  const S icpm2 = xdiv(1.0, cpm * cpm);
   S* gy = sb + VS_GY;
   if (tm.tl == 0)
-    gy[0] = Tbar - Dbar * invT + V * invT * Sp - vT * V * (cpw / cpm - T * Q * dcpm * icpm2);
+    gy[0] = Tbar - Dbar * invT + V * invT * Sp - vT * V * (xdiv(cpw, cpm) - T * Q * dcpm * icpm2);
   const S cbb = sb[VS_CB + BATH];
   const S cpb = sb[VS_CP + BATH];
   for (int j = tm.tl; j < NS - 1; j += TEAM) {
@@ -1951,7 +2313,8 @@ __device__ void vjp(const Team& tm, double P, const double* __restrict__ lnA_ext
 
 // Solve M^T x = b in place at slot ob with the LU of P M (P M = L U, so M^T = U^T L^T P):
 // U^T z = b forward, L^T t = z backward, x = P^T t.  The first warp works.
-__device__ void lu_solve_T(const Team& tm, int ob) {
+OUTLINE void lu_solve_T(int ob) {
+  const Team tm = make_team();
   if (tm.tl < 32) {
     const int ln = tm.tl;
     for (int i = ln; i < NEQ; i += 32) tm.at(AOFF_TMP, i) = tm.at(ob, i);
@@ -2012,37 +2375,37 @@ __device__ void adjoint_step(const Team& tm, double P, double h, const double* l
   const int U1 = OFF_U1, U2 = OFF_U2, U3 = OFF_U3, U4 = OFF_U4;
   const int W1 = AOFF_W, W2 = AOFF_W + NEQ, W3 = AOFF_W + 2 * NEQ, W4 = AOFF_W + 3 * NEQ;
   const int B1 = AOFF_UB, B2 = AOFF_UB + NEQ, B3 = AOFF_UB + 2 * NEQ, B4 = AOFF_UB + 3 * NEQ;
-  const double ih = 1.0 / h;
+  const double ih = fx_rcp(h);
   // ---- forward recompute
-  eval_f_jac(tm, OFF_Y, U1, P, lnA_ext, -1.0, 1.0 / (RGAM * h));
-  lu_factor(tm);
-  lu_solve_col(tm, U1);
+  eval_f_jac<-1>(OFF_Y, U1, P, lnA_ext, fx_rcp(RGAM * h));
+  lu_factor();
+  lu_solve_col(U1);
   for (int i = tm.tl; i < NEQ; i += TEAM) {
     const double v = tm.at(OFF_Y, i) + RA21 * tm.at(U1, i);
     tm.at(OFF_YT, i) = v;
     tm.at(AOFF_Y2, i) = v;
   }
   tsync();
-  eval_f(tm, OFF_YT, OFF_F, P, lnA_ext);
+  eval_f(OFF_YT, OFF_F, P, lnA_ext);
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(U2, i) = tm.at(OFF_F, i) + (RC21 * ih) * tm.at(U1, i);
   tsync();
-  lu_solve_col(tm, U2);
+  lu_solve_col(U2);
   for (int i = tm.tl; i < NEQ; i += TEAM) {
     const double v = tm.at(OFF_Y, i) + RA31 * tm.at(U1, i) + RA32 * tm.at(U2, i);
     tm.at(OFF_YT, i) = v;
     tm.at(AOFF_Y3, i) = v;
   }
   tsync();
-  eval_f(tm, OFF_YT, OFF_F, P, lnA_ext);
+  eval_f(OFF_YT, OFF_F, P, lnA_ext);
   for (int i = tm.tl; i < NEQ; i += TEAM)
     tm.at(U3, i) = tm.at(OFF_F, i) + (RC31 * ih) * tm.at(U1, i) + (RC32 * ih) * tm.at(U2, i);
   tsync();
-  lu_solve_col(tm, U3);
+  lu_solve_col(U3);
   for (int i = tm.tl; i < NEQ; i += TEAM)
     tm.at(U4, i) = tm.at(OFF_F, i) + (RC41 * ih) * tm.at(U1, i) + (RC42 * ih) * tm.at(U2, i) +
                    (RC43 * ih) * tm.at(U3, i);
   tsync();
-  lu_solve_col(tm, U4);
+  lu_solve_col(U4);
   // ---- reverse
   for (int i = tm.tl; i < NEQ; i += TEAM) {
     const double l = tm.at(AOFF_LAM, i);
@@ -2056,7 +2419,7 @@ __device__ void adjoint_step(const Team& tm, double P, double h, const double* l
   // stage 4
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(W4, i) = tm.at(B4, i);
   tsync();
-  lu_solve_T(tm, W4);
+  lu_solve_T(W4);
   for (int i = tm.tl; i < NEQ; i += TEAM) {
     const double w = tm.at(W4, i);
     tm.at(AOFF_FB, i) = w;
@@ -2068,7 +2431,7 @@ __device__ void adjoint_step(const Team& tm, double P, double h, const double* l
   // stage 3
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(W3, i) = tm.at(B3, i);
   tsync();
-  lu_solve_T(tm, W3);
+  lu_solve_T(W3);
   for (int i = tm.tl; i < NEQ; i += TEAM) {
     const double w = tm.at(W3, i);
     tm.at(AOFF_FB, i) += w;
@@ -2078,12 +2441,12 @@ __device__ void adjoint_step(const Team& tm, double P, double h, const double* l
   }
   tsync();
   set_vjp_state<double>(tm, AOFF_Y3, AOFF_Y3);
-  vjp<double>(tm, P, lnA_ext);
+  vjp<double>(P, lnA_ext);
   add_gy(tm, false, AOFF_YB, 1.0, B1, RA31, B2, RA32);
   // stage 2
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(W2, i) = tm.at(B2, i);
   tsync();
-  lu_solve_T(tm, W2);
+  lu_solve_T(W2);
   for (int i = tm.tl; i < NEQ; i += TEAM) {
     const double w = tm.at(W2, i);
     tm.at(AOFF_V, i) = w;
@@ -2091,23 +2454,23 @@ __device__ void adjoint_step(const Team& tm, double P, double h, const double* l
   }
   tsync();
   set_vjp_state<double>(tm, AOFF_Y2, AOFF_Y2);
-  vjp<double>(tm, P, lnA_ext);
+  vjp<double>(P, lnA_ext);
   add_gy(tm, false, AOFF_YB, 1.0, B1, RA21, -1, 0.0);
   // stage 1
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(W1, i) = tm.at(B1, i);
   tsync();
-  lu_solve_T(tm, W1);
+  lu_solve_T(W1);
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(AOFF_V, i) = tm.at(W1, i);
   tsync();
   set_vjp_state<double>(tm, OFF_Y, OFF_Y);
-  vjp<double>(tm, P, lnA_ext);
+  vjp<double>(P, lnA_ext);
   add_gy(tm, false, AOFF_YB, 1.0, -1, 0.0, -1, 0.0);
   // M = I/(gamma h) - J(y): second-order terms along each u_i with weights w_i
   for (int st = 0; st < 4; ++st) {
     for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(AOFF_V, i) = tm.at(AOFF_W + st * NEQ, i);
     tsync();
     set_vjp_state<DD>(tm, OFF_Y, UOFF(st));
-    vjp<DD>(tm, P, lnA_ext);
+    vjp<DD>(P, lnA_ext);
     add_gy(tm, true, AOFF_YB, 1.0, -1, 0.0, -1, 0.0);
   }
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.at(AOFF_LAM, i) = tm.at(AOFF_YB, i);
@@ -2136,8 +2499,7 @@ chem_adjoint_k(long long n_cells, const double* __restrict__ P, const double* __
                const int* __restrict__ tape_nacc, const double* __restrict__ tape_h,
                const double* __restrict__ tape_ck, int interval, double* __restrict__ seg,
                double* __restrict__ gp_partial, unsigned long long* queue) {
-  extern __shared__ double smem[];
-  const Team tm = make_team(smem);
+  const Team tm = make_team();
   const long long tg = team_global_id();
   for (int r = tm.tl; r < NR; r += TEAM) tm.at(AOFF_GP, r) = 0.0;
   tsync();
@@ -2198,8 +2560,7 @@ extern "C" __global__ void __launch_bounds__(TPB)
 chem_eval_vjp_k(long long n_cells, const double* __restrict__ T, const double* __restrict__ P,
                 const double* __restrict__ n, const double* __restrict__ v, double* __restrict__ gy,
                 double* __restrict__ gp, long long ld, const double* __restrict__ lnA_ext) {
-  extern __shared__ double smem[];
-  const Team tm = make_team(smem);
+  const Team tm = make_team();
   const long long stride = (long long)gridDim.x * NTEAM;
   for (long long c = team_global_id(); c < n_cells; c += stride) {
     if (tm.tl == 0) tm.at(OFF_Y, 0) = T[c];
@@ -2208,7 +2569,7 @@ chem_eval_vjp_k(long long n_cells, const double* __restrict__ T, const double* _
     for (int r = tm.tl; r < NR; r += TEAM) tm.at(AOFF_GP, r) = 0.0;
     tsync();
     set_vjp_state<double>(tm, OFF_Y, OFF_Y);
-    vjp<double>(tm, P[c], lnA_ext);
+    vjp<double>(P[c], lnA_ext);
     const double* g = reinterpret_cast<const double*>(&tm.base[AOFF_S]) + VS_GY;
     for (int i = tm.tl; i < NEQ; i += TEAM) gy[i * ld + c] = g[i];
     for (int r = tm.tl; r < NR; r += TEAM) gp[(long long)mk_rorig[r] * ld + c] = tm.at(AOFF_GP, r);
