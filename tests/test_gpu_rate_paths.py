@@ -11,11 +11,11 @@ pytestmark = pytest.mark.gpu
 
 EXTRA = """R ELEM 2 H 2 O 1 1 H2O 1 1.0e15 -0.5 100.0
 R ELEM 2 H 2 H2O 1 2 H2 1 H2O 1 6.0e15 -1.2 0.0
-R ELEM 1 OH 2 2 O 1 H2O 1 4.0e9 1.1 500.0
+R ELEM 1 HO 2 2 O 1 H2O 1 4.0e9 1.1 500.0
 R ELEM 1 O 3 2 O2 1 O 1 1.0e14 0.0 0.0
-R THIRD 1 OH 2 1 H2O2 1 2.0e15 -0.7 0.0
+R THIRD 1 HO 2 1 H2O2 1 2.0e15 -0.7 0.0
 EFF 2 H2O 6.0 H 2.5
-R LIND 1 OH 2 1 H2O2 1 7.0e12 -0.4 0.0
+R LIND 1 HO 2 1 H2O2 1 7.0e12 -0.4 0.0
 EFF 1 N2 0.7
 LOW 2.0e17 -0.9 -1500.0
 """
