@@ -142,6 +142,14 @@
 #else
 #define RSPLIT 1
 #endif
+#define LU_MIN 33
+// the blocked LU: a row (and a column) of the matrix per lane, and room for its exchanges in the
+// five thermo slots; smaller systems and narrower teams take the column-by-column form
+#if TEAM >= 32 && NEQ <= TEAM && NEQ >= LU_MIN && 22 * ((NEQ + 31) / 32 + 1) + 8 <= 5 * NS
+#define LU_BLOCKED 1
+#else
+#define LU_BLOCKED 0
+#endif
 // the blocked stage solves: RSPLIT lanes per row of the matrix
 #if TEAM >= 32 && NEQ <= TEAM
 #define SOLVE_BLK 1
@@ -1018,45 +1026,244 @@ OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double 
 
 // ------------------------------------------------------------------------------ LU + solves
 
-#if TEAM >= 128
-// Look-ahead part of the multi-warp LU, run by the team's first warp: column c (rows c..N-1)
-// receives the rank-1 update of step c-1 (c > 0), then its pivot (largest |a|, lowest row on
-// ties) and the pivot's inverse go to the team's scratch slots LU_PIV / LU_INV.
-#define LU_INV (OFF_RED + 21)
-#define LU_PIV (OFF_RED + 22)
-__device__ __forceinline__ void lu_panel(const Team& tm, int c) {
-  long long best = -1;
-  int p = NEQ;
-  const double u = c > 0 ? tm.A(c - 1, c) : 0.0;
-  for (int i = c + tm.tl; i < NEQ; i += 32) {
-    double a = tm.A(i, c);
-    if (c > 0) {
-      a = fma(-tm.A(i, c - 1), u, a);
-      tm.A(i, c) = a;
+#if LU_BLOCKED
+// ---- blocked LU: panels of eight columns in FP64, the trailing update on the tensor cores.
+//
+// The rank-8 update C -= L U (L m x 8, U 8 x m) is 8 m^2 FP64 FMAs: nearly all of the
+// factorisation's work, and the FP64 pipe gives a warp one per 64 clocks.  Here it is computed as
+// an integer product: every row of L and column of U is scaled by a power of two, rounded to 61 bits
+// and cut into LU_SL signed digits of nine bits, which fp16 holds exactly; mma.sync accumulates the
+// digit products of equal weight in FP32 without rounding (at most 56 products of 2^16, offset by
+// 1.5 2^23 so that the sums can be read off the bit patterns); the sums are put together in a 64-bit
+// integer (2^-60 of the largest product), rounded once to a double and subtracted from C: one FP64
+// add in place of eight FMAs, and one rounding in place of eight.
+// To keep the scaling from losing small products, U's rows are first brought to a common
+// magnitude and L's columns scaled inversely (rates of very different species meet in a panel).
+// The solutions' errors in the solver's weighted norm, against 160-bit arithmetic on 53- and
+// 111-species iteration matrices (steps of 1e-9 to 1e-6 s), are those of the FP64 update.
+#define LU_SL 7
+#define LU_NB 8
+#define LU_NW ((NEQ + 31) / 32)  // warps of the panel factorisation, one row per lane
+// scratch in the thermo slots (dead during the factorisation): two sets of candidate rows
+// (eight values, 1/pivot, key and position), one per warp and the panel's top row, then eight pivot rows
+// and the magnitudes of U's eight rows
+#define LUS_ROW(set, w) (OFF_C + ((set) * (LU_NW + 1) + (w)) * 11)
+#define LUS_INT (OFF_C + 2 * (LU_NW + 1) * 11)
+
+__device__ __forceinline__ void lu_bar() {
+#if LU_NW == 1
+  __syncwarp();
+#elif LU_NW * 32 == TEAM
+  __syncthreads();
+#else
+  asm volatile("bar.sync 1, %0;" ::"r"(LU_NW * 32) : "memory");
+#endif
+}
+
+// Columns k0..k0+kb-1, rows k0..N-1, by LU_NW warps with a row per lane in registers: per column a
+// warp argmax (three reductions), one exchange of the warps' candidates through shared memory (the
+// candidate's whole row and its reciprocal with it), and the rank-1 update of the panel.
+__device__ __forceinline__ void lu_panel8(const Team& tm, int k0) {
+  const int kb = NEQ - k0 < LU_NB ? NEQ - k0 : LU_NB;
+  const int m = NEQ - k0, w = tm.tl >> 5;
+  const bool in = tm.tl < m;
+  double v[LU_NB];
+#pragma unroll
+  for (int c = 0; c < LU_NB; ++c) v[c] = in && c < kb ? tm.A(k0 + tm.tl, k0 + c) : 0.0;
+  int* ints = reinterpret_cast<int*>(&tm.base[LUS_INT]);
+  if (tm.tl < LU_NB) ints[LU_NB + tm.tl] = 0;
+#pragma unroll
+  for (int j = 0; j < LU_NB; ++j) {
+    if (j < kb) {
+      const bool cand = in && tm.tl >= j;
+      // every lane's reciprocal, while the reductions wait; the chosen lane redoes an exceptional one
+      double inv = fx_rcp_normal(v[j]);
+      const unsigned long long key = (unsigned long long)abs_key(v[j]);
+      const unsigned hi = cand ? (unsigned)(key >> 32) : 0u, lo = cand ? (unsigned)key : 0u;
+      const unsigned mhi = __reduce_max_sync(0xffffffffu, hi);
+      const unsigned mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? lo : 0u);
+      const unsigned pos = __reduce_min_sync(0xffffffffu, cand && hi == mhi && lo == mlo ? (unsigned)tm.tl : 0xffffu);
+      double* mine = &tm.base[LUS_ROW(j & 1, w)];
+      if ((unsigned)tm.tl == pos) {
+#pragma unroll
+        for (int c = 0; c < LU_NB; ++c) mine[c] = v[c];
+        if (!fx_rcp_ok(v[j])) inv = fx_rcp_slow(v[j]);
+        mine[8] = inv;
+      }
+      if ((tm.tl & 31) == 0) {
+        mine[9] = __longlong_as_double(((long long)mhi << 32) | mlo);
+        mine[10] = __longlong_as_double((long long)pos);
+      }
+      double* top = &tm.base[LUS_ROW(j & 1, LU_NW)];
+      if (tm.tl == j) {
+#pragma unroll
+        for (int c = 0; c < LU_NB; ++c) top[c] = v[c];
+      }
+      lu_bar();
+      // the winner: the largest key, the lowest position on ties (warps hold ascending positions; a
+      // warp without a candidate has position 0xffff)
+      const double* best = &tm.base[LUS_ROW(j & 1, 0)];
+      long long ck[LU_NW];
+      unsigned cp[LU_NW];
+#pragma unroll
+      for (int x = 0; x < LU_NW; ++x) {
+        ck[x] = __double_as_longlong(best[x * 11 + 9]);
+        cp[x] = (unsigned)__double_as_longlong(best[x * 11 + 10]);
+      }
+      long long bk = cp[0] != 0xffffu ? ck[0] : -1;
+      unsigned p = cp[0];
+      int bw = 0;
+#pragma unroll
+      for (int x = 1; x < LU_NW; ++x)
+        if (cp[x] != 0xffffu && ck[x] > bk) { bk = ck[x]; p = cp[x]; bw = x * 11; }
+      best += bw;
+      if ((unsigned)tm.tl == p && p != (unsigned)j) {
+#pragma unroll
+        for (int c = 0; c < LU_NB; ++c) v[c] = top[c];
+      }
+      const double pinv = best[8];
+      if (tm.tl == j) {
+#pragma unroll
+        for (int c = 0; c < LU_NB; ++c) v[c] = best[c];
+        v[j] = pinv;  // 1/U_kk on the diagonal
+        ints[j] = k0 + (int)p;
+      }
+      if (in && tm.tl > j) {
+        const double l = v[j] * pinv;
+        v[j] = l;
+#pragma unroll
+        for (int c = j + 1; c < LU_NB; ++c) v[c] = fma(-l, best[c], v[c]);
+      }
     }
-    const long long v = abs_key(a);
-    if (v > best) { best = v; p = i; }
   }
-  {
-    // warp argmax in three reductions: the high word of the key, the low word among the lanes
-    // holding that maximum, the lowest row among the lanes holding both (a lane without rows
-    // enters key 0 with row NEQ and so never wins over a row of the column)
-    const unsigned long long key = best < 0 ? 0ULL : (unsigned long long)best;
-    const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
-    const unsigned mhi = __reduce_max_sync(0xffffffffu, hi);
-    const unsigned mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? lo : 0u);
-    p = (int)__reduce_min_sync(0xffffffffu, (hi == mhi && lo == mlo) ? (unsigned)p : 0xffffffffu);
-  }
-  __syncwarp();  // the updated column is visible to the whole warp
-  const double inv = fx_rcp(tm.A(p, c));
-  if (tm.tl == 0) {
-    tm.base[LU_INV] = inv;
-    reinterpret_cast<int*>(&tm.base[LU_PIV])[0] = p;
+#pragma unroll
+  for (int c = 0; c < LU_NB; ++c)
+    if (in && c < kb) tm.A(k0 + tm.tl, k0 + c) = v[c];
+}
+
+// magnitude of x as a biased exponent (0: zero or denormal, taken as zero below)
+__device__ __forceinline__ int lu_mag(double x) { return (int)(fx_bits(x) >> 52) & 2047; }
+
+// x 2^s as the 61-bit integer X = x 2^s / 2^(top - 1022) 2^61, where mag <= top are the biased exponents of
+// |x 2^s| and of the largest number of its row or column; the constant makes every nine-bit digit
+// of the sum an unsigned one, 256 above the signed digit it stands for
+__device__ __forceinline__ fx_u64 lu_digits(double x, int mag, int top) {
+  const fx_u64 b = fx_bits(x);
+  const fx_i64 m = mag < -4000 ? 0 : (fx_i64)fx_mant(x);
+  const int d = top - mag - 8;  // >= -8
+  fx_i64 v = d <= 0 ? m << -d : m >> (d < 63 ? d : 63);
+  if ((fx_i64)b < 0) v = -v;
+  return (fx_u64)v + 256ULL * 0x0040201008040201ULL;
+}
+// digit pairs of two elements as half2 registers, most significant first
+__device__ __forceinline__ void lu_halves(fx_u64 y0, fx_u64 y1, unsigned* h) {
+#pragma unroll
+  for (int s = 0; s < LU_SL; ++s) {
+    const int sh = 9 * (LU_SL - 1 - s);
+    const unsigned a = (unsigned)(y0 >> sh) & 511u, b = (unsigned)(y1 >> sh) & 511u;
+    const unsigned x = 0x64006400u | a | (b << 16);  // 1024 + digit + 256
+    asm("sub.f16x2 %0, %1, %2;" : "=r"(h[s]) : "r"(x), "r"(0x65006500u));  // - 1280
   }
 }
-// elements of a rank-1 update that each lane of the first warp leaves to the other warps, in
-// exchange for the look-ahead column it handles
-#define LU_PANEL_SHARE 8
+__device__ __forceinline__ void lu_mma16(float* c, unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0,
+                                         unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void lu_mma8(float* c, unsigned a0, unsigned a1, unsigned b0) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(b0));
+}
+
+// The product T 2^(e - 1085) of the scaled sums as a double, T = sum_t a_t 2^(9 (5 - t)); a_t are the
+// accumulators' bit patterns (0x4b400000 + the sum).  With e the sum of the two tops less 1018 this is the
+// product of the numbers whose digits were multiplied.
+__device__ __forceinline__ double lu_value(const unsigned* a, int e) {
+  const unsigned k = 0x4b400000u;
+  const int p01 = (int)(a[0] * 512u + a[1] - k * 513u), p23 = (int)(a[2] * 512u + a[3] - k * 513u);
+  const int p45 = (int)(a[4] * 512u + a[5] - k * 513u), p6 = (int)(a[6] - k + 256u) >> 9;
+  const fx_i64 T = ((fx_i64)p01 << 36) + ((fx_i64)p23 << 18) + ((fx_i64)p45 + p6);
+  const fx_u64 sg = (fx_u64)T & 0x8000000000000000ULL;
+  const fx_u64 u = T < 0 ? 0 - (fx_u64)T : (fx_u64)T;
+  const int z = fx_clz(u);
+  const fx_u64 r = (((u << z) >> 1) + 0x200) >> 10;
+  const int ef = e - z;  // biased exponent - 1
+  if (ef <= 0 || u == 0) return 0.0;
+  return fx_as_double(sg | (ef >= 2045 ? 0x7ff0000000000000ULL : ((fx_u64)ef << 52) + r));
+}
+
+// A[k1.., k1..] -= A[k1.., k0..k0+7] A[k0..k0+7, k1..], tiles of 16 x 8 dealt to the warps in runs along a
+// strip of rows (its digits stay in registers).
+__device__ __forceinline__ void lu_update8(const Team& tm, int k0) {
+  const int k1 = k0 + LU_NB, m = NEQ - k1;
+  const int nt = (m + 7) / 8, tot = (m + 15) / 16 * nt;
+  const int ln = tm.tl & 31, w = TEAM > 32 ? tm.tl >> 5 : 0, g = ln >> 2, t = ln & 3;
+  const int* rho = reinterpret_cast<const int*>(&tm.base[LUS_INT]) + LU_NB;
+  const int rho0 = rho[2 * t], rho1 = rho[2 * t + 1];
+  int strip = -1, topl0 = 0, topl1 = 0;
+  unsigned la[LU_SL], lb[LU_SL];
+  for (int q = w * tot / (TEAM / 32); q < (w + 1) * tot / (TEAM / 32); ++q) {
+    const int s = q / nt, j0 = k1 + (q - s * nt) * 8;
+    const int r0 = k1 + s * 16 + g, r1 = r0 + 8;
+    if (s != strip) {
+      strip = s;
+      double x[4];
+      int mg[4];
+      x[0] = r0 < NEQ ? tm.A(r0, k0 + 2 * t) : 0.0;
+      x[1] = r0 < NEQ ? tm.A(r0, k0 + 2 * t + 1) : 0.0;
+      x[2] = r1 < NEQ ? tm.A(r1, k0 + 2 * t) : 0.0;
+      x[3] = r1 < NEQ ? tm.A(r1, k0 + 2 * t + 1) : 0.0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        mg[i] = lu_mag(x[i]);
+        mg[i] = mg[i] == 0 ? -8000 : mg[i] + (i & 1 ? rho1 : rho0);
+      }
+      topl0 = max(mg[0], mg[1]);
+      topl1 = max(mg[2], mg[3]);
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        topl0 = max(topl0, __shfl_xor_sync(0xffffffffu, topl0, o));
+        topl1 = max(topl1, __shfl_xor_sync(0xffffffffu, topl1, o));
+      }
+      lu_halves(lu_digits(x[0], mg[0], topl0), lu_digits(x[1], mg[1], topl0), la);
+      lu_halves(lu_digits(x[2], mg[2], topl1), lu_digits(x[3], mg[3], topl1), lb);
+    }
+    unsigned ub[LU_SL];
+    int topu;
+    {
+      const int j = j0 + g;
+      const double x0 = j < NEQ ? tm.A(k0 + 2 * t, j) : 0.0, x1 = j < NEQ ? tm.A(k0 + 2 * t + 1, j) : 0.0;
+      int m0 = lu_mag(x0), m1 = lu_mag(x1);
+      m0 = m0 == 0 ? -8000 : m0 - rho0;
+      m1 = m1 == 0 ? -8000 : m1 - rho1;
+      topu = max(m0, m1);
+      topu = max(topu, __shfl_xor_sync(0xffffffffu, topu, 1));
+      topu = max(topu, __shfl_xor_sync(0xffffffffu, topu, 2));
+      lu_halves(lu_digits(x0, m0, topu), lu_digits(x1, m1, topu), ub);
+    }
+    float acc[LU_SL][4];
+#pragma unroll
+    for (int l = 0; l < LU_SL; ++l) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[l][i] = 12582912.0f;  // 1.5 2^23
+#pragma unroll
+      for (int i = 0; i + 1 <= l; i += 2) lu_mma16(acc[l], la[i], lb[i], la[i + 1], lb[i + 1], ub[l - i], ub[l - i - 1]);
+      if ((l & 1) == 0) lu_mma8(acc[l], la[l], lb[l], ub[0]);
+    }
+    // the tops of the thread's two output columns 2t, 2t+1 (held by the lanes of those columns)
+    const int tu0 = __shfl_sync(0xffffffffu, topu, 8 * t), tu1 = __shfl_sync(0xffffffffu, topu, 8 * t + 4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = i < 2 ? r0 : r1, j = j0 + 2 * t + (i & 1);
+      unsigned a[LU_SL];
+#pragma unroll
+      for (int l = 0; l < LU_SL; ++l) a[l] = __float_as_uint(acc[l][i]);
+      if (r < NEQ && j < NEQ) tm.A(r, j) -= lu_value(a, (i < 2 ? topl0 : topl1) + (i & 1 ? tu1 : tu0) - 1018);
+    }
+  }
+}
 #endif
 
 // In-place LU with partial pivoting of A (N x N): largest |a| in the column, lowest row on
@@ -1085,69 +1292,62 @@ OUTLINE void lu_factor() {
   }
   for (int i = 0; i < NEQ; ++i) tm.perm(i) = i;
   for (int k = 0; k < NEQ; ++k) { const int p = tm.piv(k); if (p != k) { const int t = tm.perm(k); tm.perm(k) = tm.perm(p); tm.perm(p) = t; } }
-#elif TEAM >= 128
-  // Right-looking elimination with one column of look-ahead: while the team applies step k's
-  // rank-1 update to columns k+2.., the first warp updates column k+1 and finds its pivot and the
-  // pivot's inverse (lu_panel), so that the search, its reduction and the division stay off the
-  // barrier-separated critical path: two barriers per column.  Every element receives the same
-  // operations in the same order as in the column-by-column form.
+#elif LU_BLOCKED
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.perm(i) = i;
-  if (tm.tl < 32) lu_panel(tm, 0);
   tsync();
-  for (int k = 0; k < NEQ; ++k) {
-    const int p = reinterpret_cast<const int*>(&tm.base[LU_PIV])[0];
-    const double inv = tm.base[LU_INV];
-    // rows k and p exchanged (every column but k), column k below the diagonal scaled by the
-    // pivot's inverse, which replaces U_kk; the lane of row p also moves U_kk's old value
-    if (p != k)
-      for (int j = tm.tl; j < NEQ; j += TEAM)
-        if (j != k) { const double t = tm.A(k, j); tm.A(k, j) = tm.A(p, j); tm.A(p, j) = t; }
-    for (int i = k + 1 + tm.tl; i < NEQ; i += TEAM) {
-      if (i == p) {
-        const double t = tm.A(k, k);
-        tm.A(k, k) = inv;
-        tm.A(p, k) = t * inv;
-      } else {
-        tm.A(i, k) *= inv;
-      }
-    }
-    if (tm.tl == 0) {
-      if (p == k) {
-        tm.A(k, k) = inv;
-      } else {
-        const int t = tm.perm(k);
-        tm.perm(k) = tm.perm(p);
+#pragma unroll 1
+  for (int k0 = 0; k0 < NEQ; k0 += LU_NB) {
+    if (tm.tl < LU_NW * 32) lu_panel8(tm, k0);
+    tsync();
+    // the panel's row exchanges in the other columns, a lane each, and right of the panel the
+    // triangular solve U12 = L11^-1 A12
+    const int kb = NEQ - k0 < LU_NB ? NEQ - k0 : LU_NB;
+    int* ints = reinterpret_cast<int*>(&tm.base[LUS_INT]);
+    const int c = tm.tl;
+    if (c == TEAM - 1) {  // the composed permutation
+#pragma unroll 1
+      for (int i = 0; i < kb; ++i) {
+        const int p = ints[i], t = tm.perm(k0 + i);
+        tm.perm(k0 + i) = tm.perm(p);
         tm.perm(p) = t;
       }
     }
-    tsync();
-    const int m = NEQ - k - 1;
-    if (m > 0) {
-      if (tm.tl < 32) lu_panel(tm, k + 1);
-      // rank-1 update of rows k+1.., columns k+2.. (m x n2 elements in row-major order): the
-      // first warp's lanes take the first e0 of them, LU_PANEL_SHARE fewer each than the others
-      const int n2 = m - 1;
-      if (n2 > 0) {
-        const int tot = m * n2;
-        int e0 = (tot - LU_PANEL_SHARE * (TEAM - 32)) * 32 / TEAM;
-        e0 = e0 > 0 ? e0 : 0;
-        int e, st, end;
-        if (tm.tl < 32) { e = tm.tl; st = 32; end = e0; }
-        else { e = e0 + tm.tl - 32; st = TEAM - 32; end = tot; }
-        if (e < end) {
-          int i = e / n2, j = e - (e / n2) * n2;
-          const int qd = st / n2, rm = st - qd * n2;
-          for (; e < end; e += st) {
-            double& a = tm.A(k + 1 + i, k + 2 + j);
-            a = fma(-tm.A(k + 1 + i, k), tm.A(k, k + 2 + j), a);
-            i += qd;
-            j += rm;
-            if (j >= n2) { j -= n2; ++i; }
-          }
+    double u[LU_NB];
+#pragma unroll
+    for (int i = 0; i < LU_NB; ++i) u[i] = 0.0;
+    if (c < k0 || (c >= k0 + kb && c < NEQ)) {
+#pragma unroll 1
+      for (int i = 0; i < kb; ++i) {
+        const int p = ints[i];
+        if (p != k0 + i) {
+          const double a = tm.A(k0 + i, c), b = tm.A(p, c);
+          tm.A(k0 + i, c) = b;
+          tm.A(p, c) = a;
         }
       }
-      tsync();
+      if (c >= k0 + LU_NB) {
+#pragma unroll
+        for (int i = 0; i < LU_NB; ++i) u[i] = tm.A(k0 + i, c);
+#pragma unroll
+        for (int i = 1; i < LU_NB; ++i) {
+#pragma unroll
+          for (int k = 0; k < i; ++k) u[i] = fma(-tm.A(k0 + i, k0 + k), u[k], u[i]);
+        }
+#pragma unroll
+        for (int i = 1; i < LU_NB; ++i) tm.A(k0 + i, c) = u[i];
+      }
     }
+    if (k0 + LU_NB < NEQ) {
+      // the magnitudes of U's rows, which balance the update's scales
+#pragma unroll
+      for (int i = 0; i < LU_NB; ++i) {
+        const int mx = __reduce_max_sync(0xffffffffu, lu_mag(u[i]));
+        if ((tm.tl & 31) == 0 && mx > 0) atomicMax(&ints[LU_NB + i], mx);
+      }
+      tsync();
+      lu_update8(tm, k0);
+    }
+    tsync();
   }
 #else
   // the composed permutation is built as the pivots are chosen (lane 0, after the row swap's
