@@ -145,7 +145,7 @@
 #define LU_MIN 33
 // the blocked LU: a row (and a column) of the matrix per lane, and room for its exchanges in the
 // five thermo slots; smaller systems and narrower teams take the column-by-column form
-#if TEAM >= 32 && NEQ <= TEAM && NEQ >= LU_MIN && 22 * ((NEQ + 31) / 32 + 1) + 8 <= 5 * NS
+#if TEAM >= 32 && NEQ <= TEAM && NEQ >= LU_MIN && 22 * ((NEQ + 31) / 32 + 1) + 16 <= 5 * NS
 #define LU_BLOCKED 1
 #else
 #define LU_BLOCKED 0
@@ -240,6 +240,17 @@ __device__ __forceinline__ Team make_team() {
 // themselves (a pointer argument would lose its address space).
 #define OUTLINE __device__ __noinline__
 
+#if TEAM > 32
+// sum of the team's warp partials, in every lane (shuffles: log2 of the warp count FP64 adds per
+// warp, where a loop over the partials takes one each)
+__device__ __forceinline__ double warp_partials(const double* red) {
+  double v = red[threadIdx.x & (TEAM / 32 - 1)];
+#pragma unroll
+  for (int o = TEAM / 64; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+#endif
+
 // sum over the team; every lane gets the same bits (butterfly with commutative adds)
 __device__ __forceinline__ double team_sum(const Team& tm, double v) {
 #if TEAM == 1
@@ -253,8 +264,7 @@ __device__ __forceinline__ double team_sum(const Team& tm, double v) {
   __syncthreads();
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
-  v = 0.0;
-  for (int w = 0; w < TEAM / 32; ++w) v += red[w];
+  v = warp_partials(red);
   __syncthreads();
 #endif
   return v;
@@ -299,11 +309,8 @@ __device__ __forceinline__ void team_sum2(const Team& tm, double& a, double& b) 
     red[TEAM / 32 + (threadIdx.x >> 5)] = b;
   }
   __syncthreads();
-  a = b = 0.0;
-  for (int w = 0; w < TEAM / 32; ++w) {
-    a += red[w];
-    b += red[TEAM / 32 + w];
-  }
+  a = warp_partials(red);
+  b = warp_partials(red + TEAM / 32);
   __syncthreads();
 #endif
 #endif
@@ -375,8 +382,10 @@ __device__ __forceinline__ void closure_scalars(const Team& tm, double T, double
   invV = rn * (P * invT * INV_R_U);
 }
 
-template <bool WJ>
-__device__ __forceinline__ void thermo_conc(const Team& tm, int oy, double P, CellScalars& cs) {
+__device__ __noinline__ double log2_slow(double x) { return log2(x); }
+
+// WJ: with what the Jacobian needs
+__device__ __forceinline__ void thermo_conc(const Team& tm, int oy, double P, CellScalars& cs, const bool WJ) {
   const double T = tm.at(oy, 0);
   cs.T = T;
   cs.fx = fx_range(T);
@@ -388,8 +397,8 @@ __device__ __forceinline__ void thermo_conc(const Team& tm, int oy, double P, Ce
     cs.l2Tq = ((fx_i64)e << 59) + (fx_log2_mant(fx_mant(T)) >> 3);
     cs.l2T = fx_to_double(cs.l2Tq, 59);
   } else {
-    cs.invT = 1.0 / T;
-    cs.l2T = log2(T);
+    cs.invT = fx_rcp_slow(T);
+    cs.l2T = log2_slow(T);
   }
   const double invT = cs.invT, l2T = cs.l2T;
   double nb, V, invV;
@@ -501,9 +510,8 @@ struct Rate {
 
 // FP64 form, for temperatures, ln A values or falloff blends outside the fixed-point range; lKc is
 // log2 K_c.  Kept out of line: the normal path never comes here.
-template <bool WJ>
 __device__ __noinline__ void rate_fp(int r, int kind, double T, double invT, double l2T, double lA, double M,
-                                     double lKc, Rate* out) {
+                                     double lKc, const bool WJ, Rate* out) {
   const double lnT = l2T * LN2;
   const double kinf = exp(lA + mk_b[r] * lnT - mk_th[r] * invT);
   double kf = kinf;
@@ -552,46 +560,32 @@ __device__ __noinline__ void rate_fp(int r, int kind, double T, double invT, dou
   out->dlM = dlkf_dM;
 }
 
-// Fixed-point form: log2 k in Q52 as ln A / ln2 + b log2 T - (theta / ln2) / T, the falloff blend and
-// the equilibrium constant added as logarithms, one fx_exp2 for k_f and one for k_r.  An FP64
-// exp() per reaction and the products of species' exponentials for k_r took 300 + 80 clocks of an
-// SM per warp, the two integer exponentials take 60.  Returns false where the values leave the
-// fixed-point range.
+// Falloff in fixed point: the logarithm of k (less that of 1 / (1 + Pr), returned as g1) from that of
+// k_inf.
+struct Falloff {
+  fx_i64 lk;
+  double g1, dlT, dlM;
+  bool ok;
+};
 template <bool WJ>
-__device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, const longlong2 k1, fx_i64 th,
-                                        const double* __restrict__ lA_ext, double M, fx_i64 lKc, Rate* out) {
-  fx_i64 lk = k1.x;
-  if (lA_ext) {
-    const double lA = *lA_ext;
-    if (!(fabs(lA) < 500.0)) return false;
-    lk = fx_mulhi_s(fx_from_double(lA, 54), 0x5c551d94ae0bf85eLL);  // Q54 x Q62: log2 A in Q52
-  }
-  lk += fx_mulhi_s(k1.y, cs.l2Tq) - fx_mulhi_s(th, cs.iTq);
-  if (WJ) {
-    out->dlT = (mk_b[r] + mk_th[r] * cs.invT) * cs.invT;
-    out->dlM = 0.0;
-  }
-  if (kind < LIND) {
-    out->kf = fx_exp2(lk);
-    out->kr = fx_exp2(lk - lKc);
-    return true;
-  }
+__device__ __forceinline__ Falloff falloff_fx(int r, int kind, double T, double invT, fx_i64 l2Tq, fx_i64 iTq, double M,
+                                           fx_i64 lk) {
+  Falloff o;
+  o.ok = false;
   // log2 Pr = log2 k0 + log2 [M] - log2 k_inf, floored at 1e-300
   const longlong2 k2 = mk_kfx0[r][0];
-  const fx_i64 lfl = FX_LOG2_1EM300;
-  fx_i64 lPr = lfl;
+  fx_i64 lPr = FX_LOG2_1EM300;
   bool floored = true;
   if (fx_normal_pos(M)) {
-    const fx_i64 l = k2.x + fx_mulhi_s(k2.y, cs.l2Tq) - fx_mulhi_s(mk_kfx0[r][1].x, cs.iTq) + fx_log2(M) - lk;
-    if (l >= lfl) { lPr = l; floored = false; }
+    const fx_i64 l = k2.x + fx_mulhi_s(k2.y, l2Tq) - fx_mulhi_s(mk_kfx0[r][1].x, iTq) + fx_log2(M) - lk;
+    if (l >= FX_LOG2_1EM300) { lPr = l; floored = false; }
   }
-  const double g1 = fx_rcp(1.0 + fx_exp2(lPr));  // 1 / (1 + Pr)
-  lk += lPr;
+  o.g1 = fx_rcp(1.0 + fx_exp2(lPr));  // 1 / (1 + Pr)
+  o.lk = lk + lPr;
   double dlF_dlPr = 0.0, dlF_dT = 0.0;
   if (kind == TROE) {
     const double a = mk_troe[r][0];
     const double* t = mk_troe_l2[r];  // log2(e) / T***, log2(e) / T*, log2(e) T**
-    const double T = cs.T, invT = cs.invT;
     const double e3 = fx_exp2(-fx_from_double(T * t[0], 52));
     const double e1 = fx_exp2(-fx_from_double(T * t[1], 52));
     double Fc = (1.0 - a) * e3 + a * e1;
@@ -600,7 +594,7 @@ __device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, 
       e2 = fx_exp2(-fx_from_double(t[2] * invT, 52));
       Fc += e2;
     }
-    if (!fx_normal_pos(Fc)) return false;
+    if (!fx_normal_pos(Fc)) return o;
     const double lFc = fx_log2_d(Fc) * LOG10_2;
     const double n = 0.75 - 1.27 * lFc;
     const double x = fx_to_double(lPr, 52) * LOG10_2 + (-0.4 - 0.67 * lFc);
@@ -608,8 +602,8 @@ __device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, 
     const double f1 = x * id;
     const double den = fx_rcp(1.0 + f1 * f1);
     const double lF = lFc * den;
-    if (!(fabs(lF) < 100.0)) return false;
-    lk += fx_from_double(lF * LOG2_10, 52);
+    if (!(fabs(lF) < 100.0)) return o;
+    o.lk += fx_from_double(lF * LOG2_10, 52);
     if (WJ) {
       const double g2 = 2.0 * lF * f1 * den;  // -d log10F / d f1
       const double id2 = id * id;
@@ -620,13 +614,50 @@ __device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, 
       dlF_dT = (den - g2 * df1_dlFc) * dFc * fx_rcp(Fc);
     }
   }
-  out->kf = fx_exp2(lk) * g1;
-  out->kr = fx_exp2(lk - lKc) * g1;
   if (WJ) {
-    const double g = floored ? 0.0 : g1 + dlF_dlPr;
-    const double dlk0 = (mk_b0[r] + mk_th0[r] * cs.invT) * cs.invT;
-    out->dlM = floored ? 0.0 : g * fx_rcp(M);
-    out->dlT = out->dlT + g * (dlk0 - out->dlT) + dlF_dT;
+    const double dlk = (mk_b[r] + mk_th[r] * invT) * invT;
+    const double g = floored ? 0.0 : o.g1 + dlF_dlPr;
+    const double dlk0 = (mk_b0[r] + mk_th0[r] * invT) * invT;
+    o.dlM = floored ? 0.0 : g * fx_rcp(M);
+    o.dlT = dlk + g * (dlk0 - dlk) + dlF_dT;
+  }
+  o.ok = true;
+  return o;
+}
+
+// Fixed-point form: log2 k in Q52 as ln A / ln2 + b log2 T - (theta / ln2) / T, the falloff blend and
+// the equilibrium constant added as logarithms, one fx_exp2 for k_f and one for k_r.  An FP64
+// exp() per reaction and the products of species' exponentials for k_r took 300 + 80 clocks of an
+// SM per warp, the two integer exponentials take 60.  Returns false where the values leave the
+// fixed-point range.
+__device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, const longlong2 k1, fx_i64 th,
+                                        const double* __restrict__ lA_ext, double M, fx_i64 lKc, const bool WJ,
+                                        Rate& out) {
+  fx_i64 lk = k1.x;
+  if (lA_ext) {
+    const double lA = *lA_ext;
+    if (!(fabs(lA) < 500.0)) return false;
+    lk = fx_mulhi_s(fx_from_double(lA, 54), 0x5c551d94ae0bf85eLL);  // Q54 x Q62: log2 A in Q52
+  }
+  lk += fx_mulhi_s(k1.y, cs.l2Tq) - fx_mulhi_s(th, cs.iTq);
+  double g1 = 1.0;
+  out.dlM = 0.0;
+  if (kind >= LIND) {
+    const Falloff o = WJ ? falloff_fx<true>(r, kind, cs.T, cs.invT, cs.l2Tq, cs.iTq, M, lk)
+                         : falloff_fx<false>(r, kind, cs.T, cs.invT, cs.l2Tq, cs.iTq, M, lk);
+    if (!o.ok) return false;
+    lk = o.lk;
+    g1 = o.g1;
+    out.dlT = o.dlT;
+    out.dlM = o.dlM;
+  } else if (WJ) {
+    out.dlT = (mk_b[r] + mk_th[r] * cs.invT) * cs.invT;
+  }
+  out.kf = fx_exp2(lk);
+  out.kr = fx_exp2(lk - lKc);
+  if (kind >= LIND) {
+    out.kf *= g1;
+    out.kr *= g1;
   }
   return true;
 }
@@ -649,21 +680,42 @@ __device__ __forceinline__ void gather_run(const Team& tm, const uint4 g, int ds
     q[i] = (e[i] & 0x8000u) ? dneg(q[i]) : q[i];
     q[i] = (e[i] & 0x4000u) ? 0.0 : q[i];
   }
-  double v = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + q[6]);
+  // (an FP64 add costs its pipe time for one lane or all: skipped where no lane of the warp has one;
+  // teams of four and eight lanes add without asking, since a warp takes one team's vote at a time:
+  // 65,536 13-species cells at 8 lanes 12.1 -> 11.3 ms, at 16 lanes 12.8 with the votes, 13.8 without)
   const unsigned msk = team_mask();
+  double v = q[0] + q[1];
+#pragma unroll
+  for (int i = 2; i < 7; ++i)
+    if (TEAM < 16 || __any_sync(msk, !(e[i] & 0x4000u))) v += q[i];
 #pragma unroll
   for (int o = 1; o < 8 && o < WL; o <<= 1) {
-    const double w = __shfl_down_sync(msk, v, o, WL);
-    if (g.x & (256u << (o >> 1))) v += w;
+    const bool add = (g.x & (256u << (o >> 1))) != 0;
+    if (TEAM < 16 || __any_sync(msk, add)) {
+      const double w = __shfl_down_sync(msk, v, o, WL);
+      if (add) v += w;
+    }
   }
   double* p = &tm.at(dst, g.x & 255u);
   if (g.x & 0x1000u) atomicAdd(p, v);
   else if (g.x & 0x800u) *p += v;
 }
-__device__ __forceinline__ void gather_species(const Team& tm, int ch, const uint4 first, int dst) {
+#if TEAM < 16
+__device__ __forceinline__
+#else
+OUTLINE
+#endif
+void gather_species(int ch, const uint4 first, int dst) {
+  const Team tm = make_team();
   const int n = mk_osegoff[ch + 1] - mk_osegoff[ch];  // a multiple of TEAM
-  gather_run(tm, first, dst);
-  for (int sg = tm.tl + TEAM; sg < n; sg += TEAM) gather_run(tm, mk_oseg[mk_osegoff[ch] + sg], dst);
+  uint4 g = first;
+#pragma unroll 1
+  for (int sg = tm.tl;;) {
+    gather_run(tm, g, dst);
+    sg += TEAM;
+    if (sg >= n) break;
+    g = mk_oseg[mk_osegoff[ch] + sg];
+  }
 }
 
 #if GATHER_J
@@ -709,9 +761,8 @@ __device__ __forceinline__ void gather_jacobian(const Team& tm, int ch) {
 // rate constants and d q/dT in shared memory, then the team gathers them by species and by
 // Jacobian entry.  What few reactions have (third-body parts, sides of third order) and a single
 // lane's sums are added in place.
-template <bool WJ>
 __device__ __forceinline__ void reaction_loop(const Team& tm, const CellScalars& cs, double P,
-                                              const double* __restrict__ lnA_ext) {
+                                              const double* __restrict__ lnA_ext, const bool WJ) {
   const double T = cs.T, invT = cs.invT;
   const double Ctot = P * invT * INV_R_U;    // sum_k C_k = P / (R T)
 #if TEAM == 1
@@ -753,7 +804,7 @@ __device__ __forceinline__ void reaction_loop(const Team& tm, const CellScalars&
 #pragma unroll
       for (int i = 0; i < 6; ++i)
         if (nu(i)) lKc += (i < 3 ? -nu(i) : nu(i)) * (fx_i64)fx_bits(tm.at(OFF_G, sp(i)));
-      ok = rate_fx<WJ>(r, kind, cs, kf1, kf2.x, lAe, M, lKc, &q);
+      ok = rate_fx(r, kind, cs, kf1, kf2.x, lAe, M, lKc, WJ, q);
     }
     if (!ok) {
       double lKc = dnu * (LOG2_PATM_R - cs.l2T);
@@ -764,7 +815,7 @@ __device__ __forceinline__ void reaction_loop(const Team& tm, const CellScalars&
           lKc += (i < 3 ? -nu(i) : nu(i)) * (cs.fx ? fx_to_double((fx_i64)fx_bits(g), 52) : g);
         }
       Rate qs;  // (its address is taken: kept apart from the registers of the normal path)
-      rate_fp<WJ>(r, kind, T, invT, cs.l2T, lAe ? *lAe : mk_lnA[r], M, lKc, &qs);
+      rate_fp(r, kind, T, invT, cs.l2T, lAe ? *lAe : mk_lnA[r], M, lKc, WJ, &qs);
       q = qs;
     }
     double fwd = q.kf, rev = q.kr;
@@ -857,7 +908,7 @@ __device__ __forceinline__ void reaction_loop(const Team& tm, const CellScalars&
       }
     }
     tsync();
-    gather_species(tm, ch, run, OFF_OM);
+    gather_species(ch, run, OFF_OM);
     if (WJ) {
 #if GATHER_J
       gather_jacobian(tm, ch);
@@ -867,7 +918,7 @@ __device__ __forceinline__ void reaction_loop(const Team& tm, const CellScalars&
       for (int rd = 0; rd < (CHUNK + TEAM - 1) / TEAM; ++rd)
         if (rd * TEAM + tm.tl < CHUNK) tm.at(OFF_Q, rd * TEAM + tm.tl) = dqT[rd];
       tsync();
-      gather_species(tm, ch, run, OFF_DOMT);
+      gather_species(ch, run, OFF_DOMT);
     }
     tsync();
 #endif
@@ -903,26 +954,19 @@ __device__ __forceinline__ void zero_rates(const Team& tm, bool with_j) {
   tsync();
 }
 
-// f(y) into slot `of` for the state at slot `oy`.
-OUTLINE void eval_f(int oy, int of, double P, const double* lnA_ext) {
+// f(y) into slot `of` for the state at slot `oy` and, for sgn != 0, the state Jacobian into A: J for
+// sgn = 1 (shift = 0), and M = I shift - J with shift = 1/(gamma h) for sgn = -1.
+template <int sgn>
+OUTLINE void evaluate(int oy, int of, double P, const double* lnA_ext, double shift) {
   const Team tm = make_team();
   CellScalars cs;
-  thermo_conc<false>(tm, oy, P, cs);
-  zero_rates(tm, false);
-  reaction_loop<false>(tm, cs, P, lnA_ext);
-  source_from_omega(tm, cs, of);
-}
-
-// f(y) into `of` and the state Jacobian into A: J for SGN = 1 (shift = 0), and M = I shift - J with
-// shift = 1/(gamma h) for SGN = -1.
-template <int SGN>
-OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double shift) {
-  const Team tm = make_team();
-  CellScalars cs;
-  thermo_conc<true>(tm, oy, P, cs);
-  zero_rates(tm, true);
-  reaction_loop<true>(tm, cs, P, lnA_ext);
+  thermo_conc(tm, oy, P, cs, sgn != 0);
+  zero_rates(tm, sgn != 0);
+  reaction_loop(tm, cs, P, lnA_ext, sgn != 0);
   const double fT = source_from_omega(tm, cs, of);
+  if (sgn == 0) return;
+  const long long flip = sgn < 0 ? (long long)0x8000000000000000ULL : 0;
+  auto signed_by = [&](double x) { return __longlong_as_double(__double_as_longlong(x) ^ flip); };
   const double T = cs.T, V = cs.V, invT = cs.invT;
   const double Ctot = P * invT * INV_R_U;
   const double RTP = R_U * T * fx_rcp(P);  // R T / P
@@ -960,9 +1004,9 @@ OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double 
     const double al = tm.at(OFF_AL, i - 1), be = tm.at(OFF_BE, i - 1);
     for (int l = 1; l < NEQ; ++l) {
       const double w = mk_wratio[l - 1];
-      tm.A(i, l) = SGN > 0 ? (tm.A(i, l) + be) - w * al : w * al - (tm.A(i, l) + be);
+      tm.A(i, l) = signed_by(fma(-w, al, tm.A(i, l) + be));
     }
-    tm.A(i, 0) = SGN > 0 ? tm.at(OFF_JT, i - 1) : dneg(tm.at(OFF_JT, i - 1));
+    tm.A(i, 0) = signed_by(tm.at(OFF_JT, i - 1));
   }
 #else
   {
@@ -970,10 +1014,10 @@ OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double 
     for (int e = tm.tl; e < (NEQ - 1) * NEQ; e += TEAM) {
       const int k = i - 1;
       if (l == 0) {
-        tm.A(i, 0) = SGN > 0 ? tm.at(OFF_JT, k) : dneg(tm.at(OFF_JT, k));
+        tm.A(i, 0) = signed_by(tm.at(OFF_JT, k));
       } else {
         const double w = mk_wratio[l - 1], al = tm.at(OFF_AL, k), a = tm.A(i, l) + tm.at(OFF_BE, k);
-        tm.A(i, l) = SGN > 0 ? a - w * al : w * al - a;
+        tm.A(i, l) = signed_by(fma(-w, al, a));
       }
       i += TEAM / NEQ;
       l += TEAM % NEQ;
@@ -1000,7 +1044,7 @@ OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double 
     }
     if (i < NEQ) s0 += tm.at(OFF_HRT, i - 1) * tm.A(i, l);
     double s = rsplit_sum(s0 + s1);
-    if (SGN < 0) s = dneg(s);  // the rows above carry the sign
+    s = signed_by(s);  // the rows above carry the sign
     if (ll < NEQ && tm.tl % RSPLIT == 0) {
       double val;
       if (l == 0) {
@@ -1014,14 +1058,22 @@ OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double 
         const double dcpm = tm.at(OFF_CP, l - 1) - w * tm.at(OFF_CP, BATH);
         val = -(T * s + fT * dcpm) * icpm;
       }
-      tm.A(0, l) = SGN > 0 ? val : dneg(val);
+      tm.A(0, l) = signed_by(val);
     }
   }
   tsync();
-  if (SGN < 0) {
+  if (sgn < 0) {
     for (int i = tm.tl; i < NEQ; i += TEAM) tm.A(i, i) += shift;
     tsync();
   }
+}
+
+__device__ __forceinline__ void eval_f(int oy, int of, double P, const double* lnA_ext) {
+  evaluate<0>(oy, of, P, lnA_ext, 0.0);
+}
+template <int SGN>
+__device__ __forceinline__ void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double shift) {
+  evaluate<SGN>(oy, of, P, lnA_ext, shift);
 }
 
 // ------------------------------------------------------------------------------ LU + solves
@@ -1045,10 +1097,10 @@ OUTLINE void eval_f_jac(int oy, int of, double P, const double* lnA_ext, double 
 #define LU_NB 8
 #define LU_NW ((NEQ + 31) / 32)  // warps of the panel factorisation, one row per lane
 // scratch in the thermo slots (dead during the factorisation): two sets of candidate rows
-// (eight values, 1/pivot, key and position), one per warp and the panel's top row, then eight pivot rows
-// and the magnitudes of U's eight rows
+// (eight values, 1/pivot, key and position), one per warp and the panel's top row, then, for two
+// panels in turn, eight pivot rows and the magnitudes of U's eight rows
 #define LUS_ROW(set, w) (OFF_C + ((set) * (LU_NW + 1) + (w)) * 11)
-#define LUS_INT (OFF_C + 2 * (LU_NW + 1) * 11)
+#define LUS_INT(k0) (OFF_C + 2 * (LU_NW + 1) * 11 + ((k0) / LU_NB & 1) * 8)
 
 __device__ __forceinline__ void lu_bar() {
 #if LU_NW == 1
@@ -1070,7 +1122,7 @@ __device__ __forceinline__ void lu_panel8(const Team& tm, int k0) {
   double v[LU_NB];
 #pragma unroll
   for (int c = 0; c < LU_NB; ++c) v[c] = in && c < kb ? tm.A(k0 + tm.tl, k0 + c) : 0.0;
-  int* ints = reinterpret_cast<int*>(&tm.base[LUS_INT]);
+  int* ints = reinterpret_cast<int*>(&tm.base[LUS_INT(k0)]);
   if (tm.tl < LU_NB) ints[LU_NB + tm.tl] = 0;
 #pragma unroll
   for (int j = 0; j < LU_NB; ++j) {
@@ -1194,18 +1246,21 @@ __device__ __forceinline__ double lu_value(const unsigned* a, int e) {
   return fx_as_double(sg | (ef >= 2045 ? 0x7ff0000000000000ULL : ((fx_u64)ef << 52) + r));
 }
 
-// A[k1.., k1..] -= A[k1.., k0..k0+7] A[k0..k0+7, k1..], tiles of 16 x 8 dealt to the warps in runs along a
-// strip of rows (its digits stay in registers).
-__device__ __forceinline__ void lu_update8(const Team& tm, int k0) {
+// A[k1.., k1..] -= A[k1.., k0..k0+7] A[k0..k0+7, k1..] for the column tiles c0..c1-1 (of eight columns), by
+// warp w of nw: tiles of 16 x 8 are dealt to the warps in runs along a strip of rows (its digits stay
+// in registers).
+__device__ __forceinline__ void lu_update8(const Team& tm, int k0, int w, int nw, int c0, int c1) {
   const int k1 = k0 + LU_NB, m = NEQ - k1;
-  const int nt = (m + 7) / 8, tot = (m + 15) / 16 * nt;
-  const int ln = tm.tl & 31, w = TEAM > 32 ? tm.tl >> 5 : 0, g = ln >> 2, t = ln & 3;
-  const int* rho = reinterpret_cast<const int*>(&tm.base[LUS_INT]) + LU_NB;
+  const int nt = c1 - c0, tot = (m + 15) / 16 * nt;
+  const int ln = tm.tl & 31, g = ln >> 2, t = ln & 3;
+  const int* rho = reinterpret_cast<const int*>(&tm.base[LUS_INT(k0)]) + LU_NB;
   const int rho0 = rho[2 * t], rho1 = rho[2 * t + 1];
   int strip = -1, topl0 = 0, topl1 = 0;
   unsigned la[LU_SL], lb[LU_SL];
-  for (int q = w * tot / (TEAM / 32); q < (w + 1) * tot / (TEAM / 32); ++q) {
-    const int s = q / nt, j0 = k1 + (q - s * nt) * 8;
+  const int q1 = (w + 1) * tot / nw;
+#pragma unroll 1
+  for (int q = w * tot / nw; q < q1; ++q) {
+    const int s = q / nt, j0 = k1 + (c0 + q - s * nt) * 8;
     const int r0 = k1 + s * 16 + g, r1 = r0 + 8;
     if (s != strip) {
       strip = s;
@@ -1295,49 +1350,51 @@ OUTLINE void lu_factor() {
 #elif LU_BLOCKED
   for (int i = tm.tl; i < NEQ; i += TEAM) tm.perm(i) = i;
   tsync();
+  // Per panel: its row exchanges and U12 in the other columns, then its update of the trailing matrix
+  // and the next panel.  Teams with more warps than a panel needs take the two together: the panel's
+  // warps update its eight columns and factor them while the others update the rest.
 #pragma unroll 1
-  for (int k0 = 0; k0 < NEQ; k0 += LU_NB) {
-    if (tm.tl < LU_NW * 32) lu_panel8(tm, k0);
-    tsync();
-    // the panel's row exchanges in the other columns, a lane each, and right of the panel the
-    // triangular solve U12 = L11^-1 A12
-    const int kb = NEQ - k0 < LU_NB ? NEQ - k0 : LU_NB;
-    int* ints = reinterpret_cast<int*>(&tm.base[LUS_INT]);
-    const int c = tm.tl;
-    if (c == TEAM - 1) {  // the composed permutation
+  for (int k0 = -LU_NB;; k0 += LU_NB) {
+    if (k0 >= 0) {
+      // the panel's row exchanges in the other columns, a lane each, and right of the panel the
+      // triangular solve U12 = L11^-1 A12
+      const int kb = NEQ - k0 < LU_NB ? NEQ - k0 : LU_NB;
+      int* ints = reinterpret_cast<int*>(&tm.base[LUS_INT(k0)]);
+      const int c = tm.tl;
+      if (c == TEAM - 1) {  // the composed permutation
 #pragma unroll 1
-      for (int i = 0; i < kb; ++i) {
-        const int p = ints[i], t = tm.perm(k0 + i);
-        tm.perm(k0 + i) = tm.perm(p);
-        tm.perm(p) = t;
-      }
-    }
-    double u[LU_NB];
-#pragma unroll
-    for (int i = 0; i < LU_NB; ++i) u[i] = 0.0;
-    if (c < k0 || (c >= k0 + kb && c < NEQ)) {
-#pragma unroll 1
-      for (int i = 0; i < kb; ++i) {
-        const int p = ints[i];
-        if (p != k0 + i) {
-          const double a = tm.A(k0 + i, c), b = tm.A(p, c);
-          tm.A(k0 + i, c) = b;
-          tm.A(p, c) = a;
+        for (int i = 0; i < kb; ++i) {
+          const int p = ints[i], t = tm.perm(k0 + i);
+          tm.perm(k0 + i) = tm.perm(p);
+          tm.perm(p) = t;
         }
       }
-      if (c >= k0 + LU_NB) {
+      double u[LU_NB];
 #pragma unroll
-        for (int i = 0; i < LU_NB; ++i) u[i] = tm.A(k0 + i, c);
-#pragma unroll
-        for (int i = 1; i < LU_NB; ++i) {
-#pragma unroll
-          for (int k = 0; k < i; ++k) u[i] = fma(-tm.A(k0 + i, k0 + k), u[k], u[i]);
+      for (int i = 0; i < LU_NB; ++i) u[i] = 0.0;
+      if (c < k0 || (c >= k0 + kb && c < NEQ)) {
+#pragma unroll 1
+        for (int i = 0; i < kb; ++i) {
+          const int p = ints[i];
+          if (p != k0 + i) {
+            const double a = tm.A(k0 + i, c), b = tm.A(p, c);
+            tm.A(k0 + i, c) = b;
+            tm.A(p, c) = a;
+          }
         }
+        if (c >= k0 + LU_NB) {
 #pragma unroll
-        for (int i = 1; i < LU_NB; ++i) tm.A(k0 + i, c) = u[i];
+          for (int i = 0; i < LU_NB; ++i) u[i] = tm.A(k0 + i, c);
+#pragma unroll
+          for (int i = 1; i < LU_NB; ++i) {
+#pragma unroll
+            for (int k = 0; k < i; ++k) u[i] = fma(-tm.A(k0 + i, k0 + k), u[k], u[i]);
+          }
+#pragma unroll
+          for (int i = 1; i < LU_NB; ++i) tm.A(k0 + i, c) = u[i];
+        }
       }
-    }
-    if (k0 + LU_NB < NEQ) {
+      if (k0 + LU_NB >= NEQ) break;
       // the magnitudes of U's rows, which balance the update's scales
 #pragma unroll
       for (int i = 0; i < LU_NB; ++i) {
@@ -1345,10 +1402,23 @@ OUTLINE void lu_factor() {
         if ((tm.tl & 31) == 0 && mx > 0) atomicMax(&ints[LU_NB + i], mx);
       }
       tsync();
-      lu_update8(tm, k0);
+    }
+    const int w = TEAM > 32 ? tm.tl >> 5 : 0;
+    const bool mine = w < LU_NW;  // a warp of the panel
+    const int ahead = TEAM > LU_NW * 32 ? LU_NW : 0;
+    if (k0 >= 0) {
+      const int all = (NEQ - k0 - LU_NB + 7) / 8;
+      lu_update8(tm, k0, ahead && !mine ? w - ahead : w, ahead ? (mine ? ahead : TEAM / 32 - ahead) : TEAM / 32,
+                 ahead && !mine ? 1 : 0, ahead && mine ? 1 : all);
+    }
+    if (!ahead) tsync();
+    if (mine) {
+      if (ahead) lu_bar();
+      lu_panel8(tm, k0 + LU_NB);
     }
     tsync();
   }
+  tsync();
 #else
   // the composed permutation is built as the pivots are chosen (lane 0, after the row swap's
   // barrier), so no serial pass over the pivots is needed afterwards
@@ -1974,7 +2044,8 @@ chem_eval_jacobian_k(long long n_cells, const double* __restrict__ T, const doub
 // 64-lane teams (53 species) or two 256-lane teams (111 species) per SM (GB300, 53 species
 // at seven teams: 24.2K vs 22.7K cells/s with the cap)
 // (sub-warp teams: 512 threads per SM, 128 registers a thread)
-#define MIN_BLOCKS (TEAM == 64 ? 8 : (TEAM >= 128 ? 2 : (SUBWARP ? 512 / TPB : 1)))
+#define MIN_BLOCKS \
+  (TEAM == 64 ? 8 : (TEAM >= 128 ? (TEAM == 128 && NEQ <= 64 ? 4 : 2) : (SUBWARP ? 512 / TPB : 1)))
 extern "C" __global__ void __launch_bounds__(TPB, MIN_BLOCKS)
 chem_integrate_k(long long n_cells, double* __restrict__ T, const double* __restrict__ P,
                  double* __restrict__ Y, long long ld, double dt, double rtol, double atol,
