@@ -64,7 +64,8 @@ typedef struct chem_mech* chem_mech_t;
 typedef struct {
   int32_t team;        /* lanes per cell for the default kernel config: 1 (block 32..128), 4, 8
                           or 16 (several cells per warp; block 32..128), 32 (block 32..256), 64,
-                          128, 256 (block = team); 0 = chosen from the mechanism size */
+                          128, 256 (block = team); 0 = chosen from the mechanism size and,
+                          call by call, from the number of cells */
   int32_t block;       /* threads per block; 0 = chosen with team */
   int32_t verbose;     /* print compile logs (register use) to stderr */
   const char* cache_dir; /* directory for compiled cubins; NULL = no disk cache */
@@ -96,7 +97,7 @@ typedef struct {
   double h_min;        /* smallest step size [s] before CHEM_STATUS_H_UNDERFLOW; 1e-20 */
   double T_min;        /* cells with T < T_min are skipped; 0 = none */
   int32_t mode;        /* CHEM_MODE_PERSISTENT (default) or CHEM_MODE_PLAIN */
-  int32_t team;        /* kernel config override (0 = mechanism default) */
+  int32_t team;        /* kernel config override (0 = the mechanism's; without one, by n_cells) */
   int32_t block;
   const double* lnA;   /* device [Nr]: ln of the pre-exponential factors (SI units; for falloff
                           reactions the high-pressure limit); NULL = the mechanism's values */
@@ -314,7 +315,9 @@ int chem_autotune(chem_mech_t mech, int64_t n_cells, const double* T, const doub
                   int32_t* team, int32_t* block, float* ms);
 
 /* Kernel configuration actually used by chem_integrate for these options (team, block,
- * dynamic shared memory bytes, registers per thread); for reports. */
+ * dynamic shared memory bytes, registers per thread); for reports.  Without a configuration in
+ * the options, at load or from chem_autotune it reports the mechanism's default, which calls on
+ * few cells, or of a small mechanism on many, replace by another. */
 int chem_kernel_config(chem_mech_t mech, const chem_int_opts* opts, int32_t* team,
                        int32_t* block, int32_t* smem_bytes, int32_t* regs);
 

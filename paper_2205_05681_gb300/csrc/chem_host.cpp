@@ -933,6 +933,7 @@ struct chem_mech {
   CUcontext ctx = nullptr;
   int n_sm = 0;
   int default_team = 32, default_tpb = 64;
+  bool by_cells = false;  // integrate chooses among size_configs (no configuration was asked for)
   std::mutex mu;       // guards modules
   std::mutex host_mu;  // guards the chem_integrate_host buffers
   // keyed by (lanes per cell, threads per block, Rosenbrock method)
@@ -971,6 +972,35 @@ int tstride_for(const MechData& m, int tableau, int team) {
 void default_config(int ns, int* team, int* tpb) {
   if (ns <= 64) { *team = 64; *tpb = 64; }
   else { *team = 256; *tpb = 256; }
+}
+
+// The other configurations that a call without one of its own may get, by its number of cells
+// (config_for); loaded with the mechanism, so that no call has to compile or load a module.
+std::vector<std::pair<int, int>> size_configs(int ns) {
+  if (ns <= 16) return {{16, 64}, {8, 32}};
+  if (ns <= 64) return {{128, 128}};
+  return {};
+}
+
+// Lanes per cell for n cells on n_sm SMs.  Few cells: as many lanes each as shorten its chain of
+// dependent operations; many: as few as keep the lanes busy, since a warp instruction costs its FP64
+// pipe time whatever its number of active lanes.  Measured on GB300 (152 SMs), one split step of 1 us, ms:
+//   13 species, lanes     8      16      64        53 species, lanes    64     128
+//      1,024 cells      2.11    1.32    1.15            40 cells      21.8    16.1
+//      2,000            2.12    1.41    1.45           333            26.3    20.7
+//     16,384            4.27    3.92    8.11           600            28.1    24.4
+//     30,000            6.25    6.42    14.5         1,000            35.9    39.9
+//     65,536            11.3    12.8    30.8         8,000             209     245
+// so the lines lie at 12 and 160 cells per SM (13 species) and at 4, a resident team of 128 lanes
+// each (53 species).  One evaluation of f or J (eval): the same lines for 13 species (50,000 cells, source
+// 0.20 ms at 8 lanes and 0.56 at 64); at 53 species 64 lanes win from 1,000 cells on.
+void config_for(int ns, int64_t n, int n_sm, bool eval, int* team, int* tpb) {
+  if (ns <= 16) {
+    if (n > (int64_t)160 * n_sm) { *team = 8; *tpb = 32; }
+    else if (n > (int64_t)12 * n_sm) { *team = 16; *tpb = 64; }
+  } else if (ns <= 64 && !eval) {
+    if (n <= (int64_t)4 * n_sm) { *team = 128; *tpb = 128; }
+  }
 }
 
 int check_config(int team, int tpb) {
@@ -1065,13 +1095,38 @@ int get_module(chem_mech* m, int team, int tpb, Module** out, bool adjoint = fal
   return 0;
 }
 
-int resolve(chem_mech* m, const chem_int_opts* o, Module** mod) {
+// The module of a call: the configuration asked for, else the mechanism's; for n_cells > 0 ROS4 calls
+// without one get theirs by the number of cells.
+int resolve(chem_mech* m, const chem_int_opts* o, Module** mod, int64_t n_cells = 0, bool eval = false) {
   int team = m->default_team, tpb = m->default_tpb;
   if (o && o->team > 0) {
     team = o->team;
     tpb = o->block > 0 ? o->block : (team <= 32 ? 64 : team);
+  } else if (m->by_cells && n_cells > 0 && !(o && (o->tableau != 0 || o->cell_method))) {
+    config_for((int)m->data.sp.size(), n_cells, m->n_sm, eval, &team, &tpb);
   }
   return get_module(m, team, tpb, mod, false, o ? o->tableau : 0);
+}
+
+// loads several forward configurations, compiling those that are not cached in parallel host threads
+// (NVRTC is thread-safe); the first must load, the others only if they fit
+int load_configs(chem_mech* m, const std::vector<std::pair<int, int>>& cfg) {
+  std::vector<std::string> cubins(cfg.size());
+  std::vector<std::thread> th;
+  for (size_t i = 0; i < cfg.size(); ++i)
+    th.emplace_back([&, i] {
+      std::string lg;
+      if (build_cubin(m->data, cfg[i].first, cfg[i].second, false, 0, m->cache_dir.c_str(), m->verbose, &cubins[i], &lg))
+        cubins[i].clear();
+    });
+  for (auto& t : th) t.join();
+  for (size_t i = 0; i < cfg.size(); ++i) {
+    Module* mod;
+    const int rc = get_module(m, cfg[i].first, cfg[i].second, &mod, false, 0, &cubins[i]);
+    if (rc && i == 0) return rc;
+    if (rc) m->by_cells = false;  // a configuration that does not fit: every call takes the default
+  }
+  return 0;
 }
 
 int make_current(chem_mech* m) {
@@ -1176,8 +1231,11 @@ int chem_mech_load(const char* spec_path, const chem_build_opts* opts, chem_mech
     m->default_team = opts->team;
     m->default_tpb = opts->block > 0 ? opts->block : m->default_tpb;
   }
-  Module* mod;
-  if (int rc = get_module(m.get(), m->default_team, m->default_tpb, &mod)) return rc;
+  m->by_cells = !(opts && opts->team > 0);
+  std::vector<std::pair<int, int>> cfg = {{m->default_team, m->default_tpb}};
+  if (m->by_cells)
+    for (auto& c : size_configs((int)m->data.sp.size())) cfg.push_back(c);
+  if (int rc = load_configs(m.get(), cfg)) return rc;
   CU_TRY(drv::cuMemHostAlloc((void**)&m->pinned, 64 * sizeof(unsigned), 0));
   *out = m.release();
   return 0;
@@ -1216,7 +1274,7 @@ static int eval_common(chem_mech_t m, bool jac, int64_t n_cells, const double* T
   if (!T || !P || !n || !out) return fail(CHEM_EARG, "NULL array");
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = resolve(m, nullptr, &mod)) return rc;
+  if (int rc = resolve(m, nullptr, &mod, n_cells, true)) return rc;
   long long nc = n_cells, l = ld;
   void* args[] = {&nc, (void*)&T, (void*)&P, (void*)&n, &out, &l, (void*)&lnA};
   return launch(jac ? mod->f_jac : mod->f_source, grid_for(m, mod, n_cells), mod, stream, args);
@@ -1277,7 +1335,7 @@ int chem_integrate(chem_mech_t m, int64_t n_cells, double* T, const double* P, d
   if (((uintptr_t)ws) & 255) return fail(CHEM_EARG, "workspace must be 256-byte aligned");
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = resolve(m, o, &mod)) return rc;
+  if (int rc = resolve(m, o, &mod, n_cells)) return rc;
   long long nc = n_cells, l = ld;
   CUstream s = (CUstream)stream;
   double* wjc = o ? o->jac_cache : nullptr;  // W-method factorisation cache
@@ -1891,6 +1949,7 @@ int chem_autotune(chem_mech_t m, int64_t n_cells, const double* T, const double*
   }
   drv::cuEventDestroy(e0);
   drv::cuEventDestroy(e1);
+  m->by_cells = false;  // the choice holds for every call
   m->default_team = bt;
   m->default_tpb = bb;
   if (team_out) *team_out = bt;
