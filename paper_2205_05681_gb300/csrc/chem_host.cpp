@@ -994,11 +994,13 @@ std::vector<std::pair<int, int>> size_configs(int ns) {
 // so the lines lie at 12 and 160 cells per SM (13 species) and at 4, a resident team of 128 lanes
 // each (53 species).  One evaluation of f or J (eval): the same lines for 13 species (50,000 cells, source
 // 0.20 ms at 8 lanes and 0.56 at 64); at 53 species 64 lanes win from 1,000 cells on.
-void config_for(int ns, int64_t n, int n_sm, bool eval, int* team, int* tpb) {
+enum CallKind { kIntegrate, kEval, kAdjoint };
+void config_for(int ns, int64_t n, int n_sm, CallKind kind, int* team, int* tpb) {
   if (ns <= 16) {
+    if (kind == kAdjoint) return;  // a warp per cell at least
     if (n > (int64_t)160 * n_sm) { *team = 8; *tpb = 32; }
     else if (n > (int64_t)12 * n_sm) { *team = 16; *tpb = 64; }
-  } else if (ns <= 64 && !eval) {
+  } else if (ns <= 64 && kind != kEval) {
     if (n <= (int64_t)4 * n_sm) { *team = 128; *tpb = 128; }
   }
 }
@@ -1097,13 +1099,13 @@ int get_module(chem_mech* m, int team, int tpb, Module** out, bool adjoint = fal
 
 // The module of a call: the configuration asked for, else the mechanism's; for n_cells > 0 ROS4 calls
 // without one get theirs by the number of cells.
-int resolve(chem_mech* m, const chem_int_opts* o, Module** mod, int64_t n_cells = 0, bool eval = false) {
+int resolve(chem_mech* m, const chem_int_opts* o, Module** mod, int64_t n_cells = 0, CallKind kind = kIntegrate) {
   int team = m->default_team, tpb = m->default_tpb;
   if (o && o->team > 0) {
     team = o->team;
     tpb = o->block > 0 ? o->block : (team <= 32 ? 64 : team);
   } else if (m->by_cells && n_cells > 0 && !(o && (o->tableau != 0 || o->cell_method))) {
-    config_for((int)m->data.sp.size(), n_cells, m->n_sm, eval, &team, &tpb);
+    config_for((int)m->data.sp.size(), n_cells, m->n_sm, kind, &team, &tpb);
   }
   return get_module(m, team, tpb, mod, false, o ? o->tableau : 0);
 }
@@ -1274,7 +1276,7 @@ static int eval_common(chem_mech_t m, bool jac, int64_t n_cells, const double* T
   if (!T || !P || !n || !out) return fail(CHEM_EARG, "NULL array");
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = resolve(m, nullptr, &mod, n_cells, true)) return rc;
+  if (int rc = resolve(m, nullptr, &mod, n_cells, kEval)) return rc;
   long long nc = n_cells, l = ld;
   void* args[] = {&nc, (void*)&T, (void*)&P, (void*)&n, &out, &l, (void*)&lnA};
   return launch(jac ? mod->f_jac : mod->f_source, grid_for(m, mod, n_cells), mod, stream, args);
@@ -1542,7 +1544,7 @@ int chem_integrate_ckpt(chem_mech_t m, int64_t n_cells, double* T, const double*
   int* att = o ? o->attempts : nullptr;
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = resolve(m, o, &mod)) return rc;
+  if (int rc = resolve(m, o, &mod, n_cells)) return rc;
   const TapeLayout L = tape_layout((int)m->data.sp.size(), n_cells, tape->capacity, tape->interval);
   char* b = (char*)tape->mem;
   int* tnacc = (int*)(b + L.nacc);
@@ -1565,10 +1567,10 @@ int chem_integrate_ckpt(chem_mech_t m, int64_t n_cells, double* T, const double*
   return launch(mod->f_int, grid_for(m, mod, n_cells), mod, stream, args);
 }
 
-static int adjoint_module(chem_mech_t m, const chem_int_opts* o, Module** mod) {
+static int adjoint_module(chem_mech_t m, const chem_int_opts* o, Module** mod, int64_t n_cells) {
   Module* fwd;
   if (o && o->tableau != 0) return fail(CHEM_EARG, "the adjoint is implemented for ROS4 (tableau 0)");
-  if (int rc = resolve(m, o, &fwd)) return rc;
+  if (int rc = resolve(m, o, &fwd, n_cells, kAdjoint)) return rc;
   if (fwd->team < 32) return fail(CHEM_EARG, "the adjoint needs a multi-lane configuration (team >= 32)");
   if (int rc = get_module(m, fwd->team, fwd->tpb, mod, true)) return rc;
   if (!(*mod)->f_adj)
@@ -1587,7 +1589,7 @@ size_t chem_adjoint_workspace(chem_mech_t m, int64_t n_cells, const chem_int_opt
   if (!m || n_cells < 0 || interval < 1) return 0;
   if (make_current(m)) return 0;
   Module* mod;
-  if (adjoint_module(m, o, &mod)) return 0;
+  if (adjoint_module(m, o, &mod, n_cells)) return 0;
   const int ns = (int)m->data.sp.size(), nr = (int)m->data.rx.size();
   const int64_t teams = adjoint_teams(m, mod, std::max<int64_t>(n_cells, 1));
   return 256 + align256(sizeof(double) * teams * (size_t)interval * ns) + align256(sizeof(double) * teams * nr);
@@ -1602,7 +1604,7 @@ int chem_adjoint(chem_mech_t m, int64_t n_cells, const double* P, const double* 
   if (int rc = check_tape(m, n_cells, tape)) return rc;
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = adjoint_module(m, o, &mod)) return rc;
+  if (int rc = adjoint_module(m, o, &mod, n_cells)) return rc;
   const size_t need = chem_adjoint_workspace(m, n_cells, o, tape->interval);
   if (!ws || ws_bytes < need) return fail(CHEM_EWS, "adjoint workspace of %zu bytes needed, %zu given", need, ws_bytes);
   if (((uintptr_t)ws) & 255) return fail(CHEM_EARG, "workspace must be 256-byte aligned");
@@ -1644,7 +1646,7 @@ int chem_adjoint_noalloc(chem_mech_t m, int64_t n_cells, const double* P, const 
   if (int rc = check_tape(m, n_cells, tape)) return rc;
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = adjoint_module(m, o, &mod)) return rc;
+  if (int rc = adjoint_module(m, o, &mod, n_cells)) return rc;
   {
     // set-up, once per loaded adjoint module (one per device context, made current above): the
     // device address of the module's static scratch array
@@ -1709,7 +1711,7 @@ int chem_eval_vjp(chem_mech_t m, int64_t n_cells, const double* T, const double*
   if (!T || !P || !n || !v || !gy || !gp) return fail(CHEM_EARG, "NULL array");
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = adjoint_module(m, nullptr, &mod)) return rc;
+  if (int rc = adjoint_module(m, nullptr, &mod, 0)) return rc;
   long long nc = n_cells, l = ld;
   void* args[] = {&nc, (void*)&T, (void*)&P, (void*)&n, (void*)&v, &gy, &gp, &l, (void*)&lnA};
   const int64_t tpb = teams_per_block(mod);
