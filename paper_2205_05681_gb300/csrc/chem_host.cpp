@@ -469,7 +469,7 @@ bool fx_mechanism(const MechData& m) {
 int chunk_size(int ns, int nr, int team, int stages) {
   const int room = (std::max(stages, 3) - 1) * ns / 2;
   const int c = std::max(team, room / team * team);
-  return std::min(std::min(c, 512), nr);
+  return std::max(1, std::min(std::min(c, 512), nr));
 }
 
 // both sides of at most second order: d q / d C is a coefficient times k times one concentration

@@ -72,3 +72,18 @@ def test_ln_a_outside_the_fixed_point_range(odd_mech):
     lnA[::3] -= 620.0  # beyond |ln A| = 500: these reactions take the FP64 functions
     lnA[1::3] += 0.5
     _check(om, g, st.T, st, y, lnA)
+
+
+@pytest.mark.parametrize("team,block", [(4, 64), (64, 64)])
+def test_mechanism_outside_the_fixed_point_range(odd_mech, tmp_path, team, block):
+    """An activation temperature beyond the fixed-point format: every rate takes the FP64 functions."""
+    from oracle import oracle as O
+    path, _ = odd_mech
+    text = open(path).read()
+    cold = text.replace("2 O2 1 O 1 1.0e14 0.0 0.0", "2 O2 1 O 1 1.0e14 0.0 900000.0")
+    assert cold != text
+    p = tmp_path / "cold.mech"
+    p.write_text(cold)
+    om = O.Mechanism(str(p))
+    st = states("h2_13", 24, "h2_fresh", 33)
+    _check(om, gpu_mech(str(p), team=team, block=block), st.T, st, om.state_from_TY(st.T, st.Y))
