@@ -603,7 +603,7 @@ std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, 
   o << "// generated for mechanism " << m.name << "\n";
   if (adjoint) o << "#define CHEM_ADJOINT 1\n#define CHEM_ADJ_SCRATCH_BYTES " << CHEM_ADJ_SCRATCH_BYTES << "\n";
   o << "#define NS " << ns << "\n#define NR " << nr << "\n#define TEAM " << team << "\n#define TPB " << tpb
-    << "\n#define MAXP " << kMaxSide << "\n";
+    << "\n";
   const RosCoefficients c = ros_coefficients(tableau);
   const std::vector<int> nf = stage_f_reuse(c);
   o << "#define TABLEAU_ID " << tableau << "\n#define ERK " << (c.erk ? 1 : 0) << "\n#define RS " << c.s

@@ -3,10 +3,12 @@
 // Compiled at run time by NVRTC, once per mechanism and launch configuration, after a
 // generated header (chem_host.cpp, emit_mechanism) that defines:
 //   NS, NR            species and reactions; the state length is NS ([T, n_1..n_{NS-1}])
-//   TEAM, TPB         lanes per cell (1, 32 or TPB) and threads per block
-//   MAXP              largest number of distinct species on one side of a reaction
-//   tables mk_*       NASA-7 coefficients pre-divided for cp, h and s; Arrhenius data; species
-//                     lists; efficiencies; falloff data (see emit_mechanism)
+//   TEAM, TPB         lanes per cell (1, 4, 8, 16, 32 or TPB) and threads per block
+//   CHUNK, NCHUNK     reactions per chunk of the multi-lane reaction loop, number of chunks
+//   tables mk_*       NASA-7 coefficients pre-divided for cp and h; rate constants as fixed-point
+//                     base-2 logarithms; one record per reaction; gather lists; efficiencies;
+//                     falloff data (see emit_mechanism)
+// and after fxmath.cuh (exp2, log2 and reciprocals on the integer pipe).
 //
 // What the kernels compute (Curtis, Niemeyer & Sung):
 //   * f(y), Sec. 2.1 Eq. (e:dphidt): concentrations from the unit-mass closure of Eq. (e:n_nsp);
@@ -14,7 +16,7 @@
 //     the equilibrium constant; net production rates; dT/dt from the constant-pressure energy
 //     balance;
 //   * the analytical Jacobian J = df/dy, Eq. (e:jac), in closed form: the reaction part
-//     d(omega)/dC (sparse scatter plus the dense third-body efficiency part), then the chain
+//     d(omega)/dC (sparse gather plus the dense third-body efficiency part), then the chain
 //     rule to the [T, n] state (the bath-gas column, the volume terms and the temperature row);
 //   * the transformed ROS4 step of Sec. 2.3 with partial-pivoting LU of (I/(gamma h) - J), four
 //     stage solves (three f evaluations: the Hairer-Wanner set repeats stage 3's argument for
@@ -29,8 +31,13 @@
 // warp (sub-warp teams, for small mechanisms whose loops would leave most lanes of a wider team
 // idle), contiguous arrays per team, team-masked warp synchronisation and shuffles.  TEAM == 32:
 // a warp per cell.  TEAM == TPB (64..256): a block per cell.  Reaction loops give each lane a
-// subset of reactions and scatter into the shared Jacobian with shared-memory atomics (TEAM>1).
+// subset of reactions; the team then gathers their rates by species and by Jacobian entry.
 // Every device loop is bounded; there is no grid-wide wait.
+//
+// What sets the time on GB300: an FP64 warp instruction takes 64 clocks of an SM sub-partition (16 of
+// the SM) and 64 of latency, an integer multiply 1 to 2, a tensor-core instruction 8.  So whatever is
+// not an FP64 sum or product of the state goes elsewhere: exponentials, logarithms and reciprocals
+// to the integer pipe, the LU's trailing update to the tensor cores, sums of lists to registers.
 
 #define ELEM 0
 #define THIRD 1
@@ -142,9 +149,10 @@
 #else
 #define RSPLIT 1
 #endif
-#define LU_MIN 33
 // the blocked LU: a row (and a column) of the matrix per lane, and room for its exchanges in the
-// five thermo slots; smaller systems and narrower teams take the column-by-column form
+// five thermo slots; narrower teams take the column-by-column form, and so do systems of up to 32
+// species (13 species: 19.8 K clocks against 27.8 K blocked, 53 species: 190 K against 149 K)
+#define LU_MIN 33
 #if TEAM >= 32 && NEQ <= TEAM && NEQ >= LU_MIN && 22 * ((NEQ + 31) / 32 + 1) + 16 <= 5 * NS
 #define LU_BLOCKED 1
 #else
@@ -628,8 +636,10 @@ __device__ __forceinline__ Falloff falloff_fx(int r, int kind, double T, double 
 // Fixed-point form: log2 k in Q52 as ln A / ln2 + b log2 T - (theta / ln2) / T, the falloff blend and
 // the equilibrium constant added as logarithms, one fx_exp2 for k_f and one for k_r.  An FP64
 // exp() per reaction and the products of species' exponentials for k_r took 300 + 80 clocks of an
-// SM per warp, the two integer exponentials take 60.  Returns false where the values leave the
-// fixed-point range.
+// SM per warp, the two integer exponentials take 60.  With the gathers below the source of 50,000
+// 53-species cells went from 2.91 to 1.38 ms, 37 M cells/s; what bounds it now: the falloff rounds'
+// chain (some 8,000 clocks of a Troe reaction, on one warp) and table loads from L2.  Returns
+// false where the values leave the fixed-point range.
 __device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, const longlong2 k1, fx_i64 th,
                                         const double* __restrict__ lA_ext, double M, fx_i64 lKc, const bool WJ,
                                         Rate& out) {
@@ -667,7 +677,8 @@ __device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, 
 // atomics (a compare-and-swap loop per FP64 add: 140 clocks, and as much again for every lane that
 // hits the same species).  A lane sums a run of up to seven entries of one species (a coefficient n
 // stands n times); the runs of a species lie in neighbouring lanes and are added by shuffles, and
-// the first lane stores.  A run is one 16-byte record: species (8 bits), add the value of the lane
+// the first lane stores.  A run is one 16-byte record, loaded before the barrier it waits at (the
+// lists come from L2: gathered entry by entry they took longer than the atomics): species (8 bits), add the value of the lane
 // 1, 2, 4 further (bits 8..10), store (11), by an atomic (12: more than eight runs), then seven
 // entries of position (9 bits) and sign (bit 15); bit 14: none.
 __device__ __forceinline__ void gather_run(const Team& tm, const uint4 g, int dst) {
@@ -1087,12 +1098,19 @@ __device__ __forceinline__ void eval_f_jac(int oy, int of, double P, const doubl
 // and cut into LU_SL signed digits of nine bits, which fp16 holds exactly; mma.sync accumulates the
 // digit products of equal weight in FP32 without rounding (at most 56 products of 2^16, offset by
 // 1.5 2^23 so that the sums can be read off the bit patterns); the sums are put together in a 64-bit
-// integer (2^-60 of the largest product), rounded once to a double and subtracted from C: one FP64
-// add in place of eight FMAs, and one rounding in place of eight.
+// integer, rounded once to a double and subtracted from C: one FP64 add in place of eight FMAs, and
+// one rounding in place of eight.  The digit products left out (of weight 7 and more) come to 2^-60
+// of the largest product typically and 2^-55 at most, an eighth to a hundredth of what eight
+// FP64 roundings leave.
 // To keep the scaling from losing small products, U's rows are first brought to a common
 // magnitude and L's columns scaled inversely (rates of very different species meet in a panel).
 // The solutions' errors in the solver's weighted norm, against 160-bit arithmetic on 53- and
 // 111-species iteration matrices (steps of 1e-9 to 1e-6 s), are those of the FP64 update.
+// Clocks per factorisation, column by column (with one column of look-ahead at 111 species) and in
+// this form: 53 species 190 K -> 149 K, 111 species 424 K -> 342 K, with the panel look-ahead 315 K; at
+// 13 species 20 K -> 28 K, hence LU_MIN.  What bounds it: the panel's chain (1,170 clocks a column,
+// 290 of them FP64) and, in the update, the FP64 subtractions and the recombination's integer
+// instructions (about 250 per tile of 16 x 8).
 #define LU_SL 7
 #define LU_NB 8
 #define LU_NW ((NEQ + 31) / 32)  // warps of the panel factorisation, one row per lane
@@ -1490,7 +1508,8 @@ OUTLINE void lu_factor() {
 // times per solve at 111 species.  With the 8 x 8 triangles on the diagonal inverted once per
 // factorisation (36 FP64 instructions, all triangles at once), a block takes one 8 x 8 product (two
 // products a lane and two shuffles), one barrier and eight columns' worth of independent FMAs spread
-// over RSPLIT lanes per row.  Against 160-bit arithmetic the solutions' errors are no larger than
+// over RSPLIT lanes per row: clocks per attempt in the four solves 121 K -> 70 K (53 species, few
+// cells), 230 K -> 136 K (111 species), of which the inversion takes 6 to 9 K.  Against 160-bit arithmetic the solutions' errors are no larger than
 // those of the plain substitution (geometric mean of their ratio 0.72 on 53- and 111-species
 // iteration matrices).
 #define NBK ((NEQ + 7) / 8)
