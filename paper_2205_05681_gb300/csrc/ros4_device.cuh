@@ -1827,6 +1827,7 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
 #endif
       }
       if (tm.tl == 0) { wc[WC_H] = hh; wc[WC_AGE] = 0.0; }
+      tsync();  // copied by every lane before lu_invert overwrites the diagonal blocks
     }
   }
 #if SOLVE_BLK
