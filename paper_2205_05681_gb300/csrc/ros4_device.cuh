@@ -344,10 +344,11 @@ __device__ __forceinline__ void scatter_add(double* p, double v) {
 #endif
 }
 
-// sum over the RSPLIT adjacent lanes of a row
+// sum over the RSPLIT adjacent lanes of a row (they are of one team, whose lanes alone take part: the
+// other teams of a warp are at their own cells)
 __device__ __forceinline__ double rsplit_sum(double v) {
 #pragma unroll
-  for (int o = RSPLIT / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  for (int o = RSPLIT / 2; o > 0; o >>= 1) v += __shfl_xor_sync(team_mask(), v, o);
   return v;
 }
 

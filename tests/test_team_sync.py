@@ -49,3 +49,36 @@ def test_cached_factors_are_those_of_the_iteration_matrix(emit, omech, tmp_path,
         np.fill_diagonal(U, 1.0 / np.diag(lu))
         M = np.eye(n) / (gamma * h) - J[c]
         assert np.abs(L @ U - M[perm]).max() <= 1e-12 * np.abs(M).max()
+
+
+@pytest.mark.parametrize("order", [1, -1])
+@pytest.mark.parametrize("ns,team,block", [(7, 16, 64), (2, 16, 64), (2, 8, 32), (2, 4, 32)])
+def test_teams_that_share_a_warp_wait_for_their_own_lanes_only(emit, omech, tmp_path, ns, team, block, order):
+    """Several cells per warp, with row sums split over lanes of the team (at most half as many species as
+    lanes) and a cell count that leaves the last warp's teams with different numbers of cells: no team may
+    wait for another, and f and J agree with the oracle to rounding of their largest term."""
+    from oracle import oracle as O
+    spec = TINY
+    if ns == 2:
+        spec = str(tmp_path / "h.mech")
+        with open(spec, "w") as fh:
+            fh.write(_two_species())
+    om = O.Mechanism(spec)
+    n = 2 * (block // team) + 1
+    T, P, _, y = _states(om, n, 6)
+    f, J = emulated.Emulated(tmp_path, emit, spec, team, block, emulated.EVAL).eval(T, P, y[:, 1:], om.nr, order=order)
+    fo, Jo = om.source(y, P), om.jacobian(y, P)
+    for c in range(n):
+        assert np.abs(f[c] - fo[c]).max() <= 1e-12 * np.abs(fo[c]).max()
+        assert np.abs(J[c] - Jo[c]).max() <= 1e-12 * np.abs(Jo[c]).max()
+
+
+
+def _two_species():
+    """H and H2 of the seven-species mechanism with their recombination."""
+    lines = open(TINY).read().splitlines()
+    out = ["MECHANISM h 0", "ELEMENTS H O N", "SPECIES 2"]
+    for s in ("H", "H2"):
+        i = [k for k, l in enumerate(lines) if l.startswith("SP %s " % s)][0]
+        out += lines[i:i + 3]
+    return "\n".join(out + ["REACTIONS 1", "R THIRD 1 H 2 1 H2 1 1.0e13 -0.5 0.0", "EFF 1 H2 2.0", "END", ""])
