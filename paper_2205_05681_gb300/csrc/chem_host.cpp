@@ -462,14 +462,55 @@ bool fx_mechanism(const MechData& m) {
   return true;
 }
 
+// Shared-memory slots of one cell with chunks of `chunk` reactions (0: one lane per cell); mirrors the OFF_*
+// layout of ros4_device.cuh: A, Y, YT, U1..Us, [F0], five per-species arrays, the packed permutation (and
+// pivots with one lane per cell), a chunk's net rates and, where they don't fit elsewhere, rate
+// constants, 24 reduction slots; for the adjoint kernels the AOFF_* arrays behind them.
+int cell_slots(int ns, int nr, const RosCoefficients& c, int team, int chunk, bool adjoint) {
+  const int stages = std::max(c.s, 3);  // the Jacobian assembly aliases three
+  return ns * ns + (7 + stages + (needs_f0(c) ? 1 : 0)) * ns + (ns + 1) / 2 * (team == 1 ? 2 : 1) +
+         (2 * chunk <= (stages - 1) * ns ? 1 : 3) * chunk + 24 +
+         (adjoint ? 15 * ns + nr + 2 * (11 * ns + nr + 8 * team / 32) : 0);
+}
+
+// distance in doubles between consecutive teams' slots (TSTRIDE of ros4_device.cuh): sub-warp
+// teams pad to TEAM (mod 16) so that the teams of a half-warp hit disjoint banks
+int padded_slots(int slots, int team) {
+  return team > 1 && team < 32 ? slots + (team - slots % 16 + 16) % 16 : slots;
+}
+
+// blocks per SM that the shared memory holds: 228 KB an SM, 1 KB of it reserved per block, 227 KB a block
+int shared_blocks(int slots, int team, int tpb) {
+  const int bytes = 8 * padded_slots(slots, team) * (team <= 32 ? tpb / team : 1);
+  return bytes > 227 * 1024 ? 0 : 228 * 1024 / (bytes + 1024);
+}
+
+// Register cap of the integrator's kernels as resident blocks (__launch_bounds__), so that the cells that
+// fit in shared memory can all be resident: eight 64-lane teams (53 species) or two 256-lane teams (111
+// species) per SM (GB300, 53 species at seven teams: 24.2K vs 22.7K cells/s with the cap); sub-warp
+// teams: 512 threads per SM, 128 registers a thread
+int min_blocks(int ns, int team, int tpb) {
+  if (team == 64) return 8;
+  if (team >= 128) return team == 128 && ns <= 64 ? 4 : 2;
+  return team > 1 && team < 32 ? 512 / tpb : 1;
+}
+
 // Reactions per chunk of the multi-lane kernels' reaction loop: the net rates and rate constants of
-// a chunk sit in shared memory while they are gathered per species and per Jacobian entry.  A
+// a chunk sit in shared memory while they are gathered per species and per Jacobian entry.  At best a
 // multiple of the team (one reaction per lane at least) for which the rate constants fit among the
-// stage slots that are dead then; never more than the mechanism has.
-int chunk_size(int ns, int nr, int team, int stages) {
-  const int room = (std::max(stages, 3) - 1) * ns / 2;
-  const int c = std::max(team, room / team * team);
-  return std::max(1, std::min(std::min(c, 512), nr));
+// stage slots that are dead then; never more than the mechanism has; and fewer where the chunk would
+// cost a resident block (or the configuration) that a cell without it and with one per-species array
+// more leaves room for: a chunk of as many reactions as species takes no more than that array.
+int chunk_size(int ns, int nr, const RosCoefficients& c, int team, int tpb, bool adjoint) {
+  const int room = (std::max(c.s, 3) - 1) * ns / 2;
+  int n = std::max(1, std::min(std::min(std::max(team, room / team * team), 512), nr));
+  if (team == 1) return n;
+  // blocks that the registers allow: 128 a thread without a bound of their own, the adjoint's 255
+  const int regs = adjoint ? 65536 / (256 * tpb) : std::max(min_blocks(ns, team, tpb), team == 32 ? 512 / tpb : 1);
+  const int most = std::max(1, regs);
+  const int want = std::min(most, shared_blocks(cell_slots(ns, nr, c, team, 0, adjoint) + ns, team, tpb));
+  while (n > 1 && shared_blocks(cell_slots(ns, nr, c, team, n, adjoint), team, tpb) < want) --n;
+  return n;
 }
 
 // both sides of at most second order: d q / d C is a coefficient times k times one concentration
@@ -603,7 +644,7 @@ std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, 
   o << "// generated for mechanism " << m.name << "\n";
   if (adjoint) o << "#define CHEM_ADJOINT 1\n#define CHEM_ADJ_SCRATCH_BYTES " << CHEM_ADJ_SCRATCH_BYTES << "\n";
   o << "#define NS " << ns << "\n#define NR " << nr << "\n#define TEAM " << team << "\n#define TPB " << tpb
-    << "\n";
+    << "\n#define MIN_BLOCKS " << min_blocks(ns, team, tpb) << "\n";
   const RosCoefficients c = ros_coefficients(tableau);
   const std::vector<int> nf = stage_f_reuse(c);
   o << "#define TABLEAU_ID " << tableau << "\n#define ERK " << (c.erk ? 1 : 0) << "\n#define RS " << c.s
@@ -700,7 +741,7 @@ std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, 
       << num(tr ? (double)(1.0L / (t[2] * kLn2)) : 0.0) << "," << num(tr ? (double)(t[3] / kLn2) : 0.0) << "}";
   }
   o << "};\n";
-  emit_gather(o, m, team, chunk_size(ns, nr, team, c.s));
+  emit_gather(o, m, team, chunk_size(ns, nr, c, team, tpb, adjoint));
   // one record per reaction (layout: reaction_loop)
   o << "__device__ const int4 mk_rec[" << nr << "] = {";
   for (int r = 0; r < nr; ++r) {
@@ -947,24 +988,15 @@ struct chem_mech {
 
 namespace {
 
-// shared-memory slots of one cell; mirrors the OFF_* layout of ros4_device.cuh: A, Y, YT, U1..Us, [F0], five per-species arrays, the packed permutation (and pivots with one lane per
-// cell), a chunk's net rates and, where they don't fit elsewhere, rate constants, 24 reduction slots
-int slots_for(const MechData& m, int tableau, int team) {
-  const int ns = (int)m.sp.size();
+// shared-memory slots of one cell of a module's forward kernels
+int slots_for(const MechData& m, int tableau, int team, int tpb, bool adjoint = false) {
+  const int ns = (int)m.sp.size(), nr = (int)m.rx.size();
   const RosCoefficients c = ros_coefficients(tableau);
-  const int packed = (ns + 1) / 2;
-  const int stages = std::max(c.s, 3);  // the Jacobian assembly aliases three
-  const int chunk = team == 1 ? 0 : chunk_size(ns, (int)m.rx.size(), team, c.s);
-  return ns * ns + (7 + stages + (needs_f0(c) ? 1 : 0)) * ns + packed * (team == 1 ? 2 : 1) +
-         (2 * chunk <= (stages - 1) * ns ? 1 : 3) * chunk + 24;
+  return cell_slots(ns, nr, c, team, team == 1 ? 0 : chunk_size(ns, nr, c, team, tpb, adjoint), false);
 }
 
-// distance in doubles between consecutive teams' slots (TSTRIDE of ros4_device.cuh): sub-warp
-// teams pad to TEAM (mod 16) so that the teams of a half-warp hit disjoint banks
-int tstride_for(const MechData& m, int tableau, int team) {
-  const int sl = slots_for(m, tableau, team);
-  if (team > 1 && team < 32) return sl + ((team - sl % 16 + 16) % 16);
-  return sl;
+int tstride_for(const MechData& m, int tableau, int team, int tpb, bool adjoint = false) {
+  return padded_slots(slots_for(m, tableau, team, tpb, adjoint), team);
 }
 
 // default kernel configuration by mechanism size (the autotuner's usual pick on GB300):
@@ -1013,9 +1045,9 @@ int check_config(int team, int tpb) {
   return fail(CHEM_EARG, "unsupported kernel config team=%d block=%d", team, tpb);
 }
 
-int smem_bytes(const MechData& m, int team, int tpb, int tableau) {
+int smem_bytes(const MechData& m, int team, int tpb, int tableau, bool adjoint = false) {
   const int teams = team <= 32 ? tpb / team : 1;
-  return tstride_for(m, tableau, team) * 8 * teams;
+  return tstride_for(m, tableau, team, tpb, adjoint) * 8 * teams;
 }
 
 int get_module(chem_mech* m, int team, int tpb, Module** out, bool adjoint = false, int tableau = 0,
@@ -1027,7 +1059,7 @@ int get_module(chem_mech* m, int team, int tpb, Module** out, bool adjoint = fal
   auto it = mods.find(key);
   if (it != mods.end()) { *out = it->second.get(); return 0; }
   if (int rc = check_config(team, tpb)) return rc;
-  const int smem = smem_bytes(m->data, team, tpb, tableau);
+  const int smem = smem_bytes(m->data, team, tpb, tableau, adjoint);
   int max_optin = 0;
   CUdevice dev;
   CU_TRY(drv::cuCtxGetDevice(&dev));
@@ -1059,13 +1091,14 @@ int get_module(chem_mech* m, int team, int tpb, Module** out, bool adjoint = fal
   CU_TRY(drv::cuModuleGetGlobal(&slots_ptr, &slots_sz, mod->mod, "chem_slots"));
   int dev_slots = 0;
   CU_TRY(drv::cuMemcpyDtoH(&dev_slots, slots_ptr, sizeof(int)));
-  if (dev_slots != slots_for(m->data, tableau, team))
+  if (dev_slots != slots_for(m->data, tableau, team, tpb, adjoint))
     return fail(CHEM_ECUDA, "shared-memory layout mismatch (%d vs %d)", dev_slots,
-                slots_for(m->data, tableau, team));
+                slots_for(m->data, tableau, team, tpb, adjoint));
   CU_TRY(drv::cuModuleGetGlobal(&slots_ptr, &slots_sz, mod->mod, "chem_tstride"));
   CU_TRY(drv::cuMemcpyDtoH(&dev_slots, slots_ptr, sizeof(int)));
-  if (dev_slots != tstride_for(m->data, tableau, team))
-    return fail(CHEM_ECUDA, "team stride mismatch (%d vs %d)", dev_slots, tstride_for(m->data, tableau, team));
+  if (dev_slots != tstride_for(m->data, tableau, team, tpb, adjoint))
+    return fail(CHEM_ECUDA, "team stride mismatch (%d vs %d)", dev_slots,
+                tstride_for(m->data, tableau, team, tpb, adjoint));
   for (CUfunction f : {mod->f_source, mod->f_jac, mod->f_int, mod->f_pinit, mod->f_patt}) {
     CU_TRY(drv::cuFuncSetAttribute(f, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES, smem));
     // all of L1 as shared memory: occupancy is bounded by the cells' shared-memory footprint

@@ -4,6 +4,7 @@
 // generated header (chem_host.cpp, emit_mechanism) that defines:
 //   NS, NR            species and reactions; the state length is NS ([T, n_1..n_{NS-1}])
 //   TEAM, TPB         lanes per cell (1, 4, 8, 16, 32 or TPB) and threads per block
+//   MIN_BLOCKS        blocks per SM that the integrator's registers must leave room for
 //   CHUNK, NCHUNK     reactions per chunk of the multi-lane reaction loop, number of chunks
 //   tables mk_*       NASA-7 coefficients pre-divided for cp and h; rate constants as fixed-point
 //                     base-2 logarithms; one record per reaction; gather lists; efficiencies;
@@ -2061,12 +2062,6 @@ chem_eval_jacobian_k(long long n_cells, const double* __restrict__ T, const doub
 // Persistent driver: each team pulls cells from the queue counter and integrates them to dt.
 // With TEAM == 1 each thread refills independently (per-lane refill of retired cells); the
 // loop body is one step attempt so that lanes on different cells still execute it together.
-// Registers capped so that the cells that fit in shared memory can all be resident: eight
-// 64-lane teams (53 species) or two 256-lane teams (111 species) per SM (GB300, 53 species
-// at seven teams: 24.2K vs 22.7K cells/s with the cap)
-// (sub-warp teams: 512 threads per SM, 128 registers a thread)
-#define MIN_BLOCKS \
-  (TEAM == 64 ? 8 : (TEAM >= 128 ? (TEAM == 128 && NEQ <= 64 ? 4 : 2) : (SUBWARP ? 512 / TPB : 1)))
 extern "C" __global__ void __launch_bounds__(TPB, MIN_BLOCKS)
 chem_integrate_k(long long n_cells, double* __restrict__ T, const double* __restrict__ P,
                  double* __restrict__ Y, long long ld, double dt, double rtol, double atol,
