@@ -261,7 +261,8 @@ int chem_adjoint(chem_mech_t mech, int64_t n_cells, const double* P, const doubl
  * output, as for chem_adjoint.
  *   - The first call for a mechanism and kernel configuration compiles and loads the adjoint
  *     module (as chem_adjoint does) and resolves the array's device address; make that first call
- *     before any stream capture.
+ *     before any stream capture.  Without a configuration, the first call (of any number of cells,
+ *     also none) loads the modules of every number of cells.
  *   - The array is shared by all calls on the same module and keeps the last call's contents:
  *     the entry point zeroes what must start at zero (the queue counter).  Calls whose work
  *     overlaps on the GPU (other streams, or chem_adjoint_noalloc enqueued twice without an

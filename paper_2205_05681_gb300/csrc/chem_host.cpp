@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <cstdarg>
@@ -974,7 +975,8 @@ struct chem_mech {
   CUcontext ctx = nullptr;
   int n_sm = 0;
   int default_team = 32, default_tpb = 64;
-  bool by_cells = false;  // integrate chooses among size_configs (no configuration was asked for)
+  std::atomic<bool> by_cells{false};  // calls choose among size_configs (no configuration was asked for) ...
+  std::atomic<bool> adj_by_cells{true};  // ... the adjoint's too
   std::mutex mu;       // guards modules
   std::mutex host_mu;  // guards the chem_integrate_host buffers
   // keyed by (lanes per cell, threads per block, Rosenbrock method)
@@ -1007,9 +1009,10 @@ void default_config(int ns, int* team, int* tpb) {
 }
 
 // The other configurations that a call without one of its own may get, by its number of cells
-// (config_for); loaded with the mechanism, so that no call has to compile or load a module.
-std::vector<std::pair<int, int>> size_configs(int ns) {
-  if (ns <= 16) return {{16, 64}, {8, 32}};
+// (config_for).  The forward ones are loaded with the mechanism, the adjoint's together at the first
+// adjoint call, so that no later call has to compile or load a module.
+std::vector<std::pair<int, int>> size_configs(int ns, bool adjoint = false) {
+  if (ns <= 16) return adjoint ? std::vector<std::pair<int, int>>{} : std::vector<std::pair<int, int>>{{16, 64}, {8, 32}};
   if (ns <= 64) return {{128, 128}};
   return {};
 }
@@ -1137,31 +1140,48 @@ int resolve(chem_mech* m, const chem_int_opts* o, Module** mod, int64_t n_cells 
   if (o && o->team > 0) {
     team = o->team;
     tpb = o->block > 0 ? o->block : (team <= 32 ? 64 : team);
-  } else if (m->by_cells && n_cells > 0 && !(o && (o->tableau != 0 || o->cell_method))) {
+  } else if (m->by_cells && n_cells > 0 && !(o && (o->tableau != 0 || o->cell_method)) &&
+             (kind != kAdjoint || m->adj_by_cells)) {
     config_for((int)m->data.sp.size(), n_cells, m->n_sm, kind, &team, &tpb);
   }
   return get_module(m, team, tpb, mod, false, o ? o->tableau : 0);
 }
 
-// loads several forward configurations, compiling those that are not cached in parallel host threads
+// loads several configurations, compiling those that are not cached in parallel host threads
 // (NVRTC is thread-safe); the first must load, the others only if they fit
-int load_configs(chem_mech* m, const std::vector<std::pair<int, int>>& cfg) {
+int load_configs(chem_mech* m, const std::vector<std::pair<int, int>>& cfg, bool adjoint = false) {
   std::vector<std::string> cubins(cfg.size());
   std::vector<std::thread> th;
   for (size_t i = 0; i < cfg.size(); ++i)
     th.emplace_back([&, i] {
       std::string lg;
-      if (build_cubin(m->data, cfg[i].first, cfg[i].second, false, 0, m->cache_dir.c_str(), m->verbose, &cubins[i], &lg))
+      if (build_cubin(m->data, cfg[i].first, cfg[i].second, adjoint, 0, m->cache_dir.c_str(), m->verbose, &cubins[i], &lg))
         cubins[i].clear();
     });
   for (auto& t : th) t.join();
   for (size_t i = 0; i < cfg.size(); ++i) {
     Module* mod;
-    const int rc = get_module(m, cfg[i].first, cfg[i].second, &mod, false, 0, &cubins[i]);
+    const int rc = get_module(m, cfg[i].first, cfg[i].second, &mod, adjoint, 0, &cubins[i]);
     if (rc && i == 0) return rc;
-    if (rc) m->by_cells = false;  // a configuration that does not fit: every call takes the default
+    // a configuration that does not fit: every call takes the default
+    if (adjoint && i > 0 && (rc || !mod->f_adj)) m->adj_by_cells = false;
+    else if (rc) m->by_cells = false;
   }
   return 0;
+}
+
+// the adjoint modules that calls without a configuration of their own may get
+int load_adjoint(chem_mech* m) {
+  std::vector<std::pair<int, int>> cfg = {{m->default_team, m->default_tpb}};
+  if (m->by_cells && m->adj_by_cells)
+    for (auto& c : size_configs((int)m->data.sp.size(), true)) cfg.push_back(c);
+  {
+    std::lock_guard<std::mutex> lk(m->mu);
+    bool all = true;
+    for (auto& c : cfg) all = all && m->adj_modules.count(std::make_tuple(c.first, c.second, 0));
+    if (all) return 0;
+  }
+  return load_configs(m, cfg, true);
 }
 
 int make_current(chem_mech* m) {
@@ -1600,9 +1620,11 @@ int chem_integrate_ckpt(chem_mech_t m, int64_t n_cells, double* T, const double*
   return launch(mod->f_int, grid_for(m, mod, n_cells), mod, stream, args);
 }
 
-static int adjoint_module(chem_mech_t m, const chem_int_opts* o, Module** mod, int64_t n_cells) {
+static int adjoint_module(chem_mech_t m, const chem_int_opts* o, Module** mod, int64_t n_cells, bool every = true) {
   Module* fwd;
   if (o && o->tableau != 0) return fail(CHEM_EARG, "the adjoint is implemented for ROS4 (tableau 0)");
+  if (every && !(o && o->team > 0) && m->default_team >= 32)
+    if (int rc = load_adjoint(m)) return rc;
   if (int rc = resolve(m, o, &fwd, n_cells, kAdjoint)) return rc;
   if (fwd->team < 32) return fail(CHEM_EARG, "the adjoint needs a multi-lane configuration (team >= 32)");
   if (int rc = get_module(m, fwd->team, fwd->tpb, mod, true)) return rc;
@@ -1744,7 +1766,7 @@ int chem_eval_vjp(chem_mech_t m, int64_t n_cells, const double* T, const double*
   if (!T || !P || !n || !v || !gy || !gp) return fail(CHEM_EARG, "NULL array");
   if (int rc = make_current(m)) return rc;
   Module* mod;
-  if (int rc = adjoint_module(m, nullptr, &mod, 0)) return rc;
+  if (int rc = adjoint_module(m, nullptr, &mod, 0, false)) return rc;
   long long nc = n_cells, l = ld;
   void* args[] = {&nc, (void*)&T, (void*)&P, (void*)&n, (void*)&v, &gy, &gp, &l, (void*)&lnA};
   const int64_t tpb = teams_per_block(mod);
