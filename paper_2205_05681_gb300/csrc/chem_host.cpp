@@ -423,8 +423,11 @@ double nasa_log2_g(const double* a, int i) {
 // Whether the kernels may keep rate and equilibrium constants as Q52 logarithms (|log2| < 2048) for
 // every temperature between 256 and 8192 K (fx_range): the coefficients fit their formats and no
 // sum of them, taken with its terms' magnitudes, leaves +-1900 on a grid of temperatures (the
-// functions are smooth; a mechanism that fails takes the FP64 functions).
-bool fx_mechanism(const MechData& m) {
+// functions are smooth; a mechanism that fails takes the FP64 functions).  *margin: by how much log2 A may
+// differ from the file's before a sum could leave +-2040; reactions with a run-time ln A further off
+// take the FP64 functions.
+bool fx_mechanism(const MechData& m, double* margin) {
+  *margin = 2040.0;
   if (m.sp.size() > 65535) return false;  // 16-bit indices in mk_rec
   const double ln2 = (double)kLn2, th_max = 180000.0 * ln2;
   for (auto& x : m.rx) {
@@ -456,8 +459,10 @@ bool fx_mechanism(const MechData& m) {
       const double kinf = (std::fabs(x.lnA) + std::fabs(x.theta) / T) / ln2 + std::fabs(x.b) * l2;
       // low-pressure limit, [M] of 1e-300..1e30 after the floor, a Troe blend of 10^-100
       const double k0 = x.kind >= 2 ? (std::fabs(x.lnA0) + std::fabs(x.theta0) / T) / ln2 + std::fabs(x.b0) * l2 + 334.0 : 0.0;
-      if (!(kinf + k0 + std::fabs(kc) + std::abs(d) * 20.0 < 1900.0)) return false;
-      if (x.kind >= 2 && !(kinf + 997.0 + 334.0 + std::fabs(kc) + std::abs(d) * 20.0 < 2040.0)) return false;
+      const double sum = kinf + k0 + std::fabs(kc) + std::abs(d) * 20.0;
+      const double floored = x.kind >= 2 ? kinf + 997.0 + 334.0 + std::fabs(kc) + std::abs(d) * 20.0 : 0.0;
+      if (!(sum < 1900.0) || !(floored < 2040.0)) return false;
+      *margin = std::min(*margin, 2040.0 - std::max(sum, floored));
     }
   }
   return true;
@@ -702,8 +707,9 @@ std::string emit_mechanism(const MechData& m0, int team, int tpb, bool adjoint, 
   // rate constants as base-2 logarithms in fixed point (fxmath.cuh): {log2 A in Q52, b in Q57},
   // {theta / ln2 in Q45, the reaction's range of third-body efficiencies}; the same of the low-pressure limits; Troe exponents times log2(e)
   auto q = [](long double v, int n) { return std::to_string(llrintl(ldexpl(v, n))) + "LL"; };
-  const bool fx = fx_mechanism(m);
-  o << "#define MECH_FX " << (fx ? 1 : 0) << "\n";
+  double margin;
+  const bool fx = fx_mechanism(m, &margin);
+  o << "#define MECH_FX " << (fx ? 1 : 0) << "\n#define FX_LNA_MARGIN " << q(fx ? margin : 0.0, 51) << "\n";
   std::vector<int> off(nr + 1, 0), esp;  // non-default third-body efficiencies
   std::vector<double> eval;
   for (int r = 0; r < nr; ++r) {

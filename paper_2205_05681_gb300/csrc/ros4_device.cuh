@@ -650,6 +650,8 @@ __device__ __forceinline__ bool rate_fx(int r, int kind, const CellScalars& cs, 
     const double lA = *lA_ext;
     if (!(fabs(lA) < 500.0)) return false;
     lk = fx_mulhi_s(fx_from_double(lA, 54), 0x5c551d94ae0bf85eLL);  // Q54 x Q62: log2 A in Q52
+    const fx_i64 d = (lk >> 1) - (k1.x >> 1);  // what the mechanism's own numbers leave room for (Q51)
+    if (d > FX_LNA_MARGIN || d < -FX_LNA_MARGIN) return false;
   }
   lk += fx_mulhi_s(k1.y, cs.l2Tq) - fx_mulhi_s(th, cs.iTq);
   double g1 = 1.0;
