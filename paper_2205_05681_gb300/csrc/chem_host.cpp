@@ -445,8 +445,9 @@ bool fx_mechanism(const MechData& m, double* margin) {
         if (std::fabs(a[0]) > 60.0 || std::fabs(a[5]) > th_max) return false;
         const bool used = (a == m.sp[k].nasa[0]) ? T < 1.02 * m.sp[k].Tmid : T > 0.98 * m.sp[k].Tmid;
         if (!used) continue;
-        const double v = a[0] * l2 - a[5] / (T * ln2) + c[0] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4])));
-        if (!(std::fabs(v) < 1900.0)) return false;
+        const double poly = c[0] + T * (c[1] + T * (c[2] + T * (c[3] + T * c[4])));  // formed on its own first
+        const double v = a[0] * l2 - a[5] / (T * ln2) + poly;
+        if (!(std::fabs(v) < 1900.0) || !(std::fabs(poly) < 1900.0)) return false;
         if (std::fabs(v) > std::fabs(mx)) mx = v;
       }
       g[k] = mx;
