@@ -9,7 +9,7 @@
 // Fixed-point formats are written Qn: an integer v stands for v 2^-n.
 //   fx_exp2(lg)      2^lg of a Q52 logarithm (|lg| < 2048)
 //   fx_log2(x)       log2 of a positive normal double, Q52
-//   fx_rcp(x)        1/x of any double (denormal and extreme arguments by the division)
+//   fx_rcp(x)        1/x of any double (denormal and extreme arguments by the division); fx_div(a, b) a/b
 //   fx_exp, fx_log   drop-in forms of exp and log for doubles
 // Methods: 2^(n + i/64 + s/64) = 2^n T_i (1 + p(s)) with T_i = 2^(i/64) tabulated to 64 bits and p the
 // Taylor polynomial of 2^(s/64) - 1 to degree 6 (remainder below 2^-58); log2 m = -log2 c_i +
@@ -187,6 +187,9 @@ FX_FN double fx_rcp_normal(double x) {
   return fx_as_double((b & 0x8000000000000000ULL) | (((fx_u64)(2044 - be) << 52) + r));
 }
 FX_FN double fx_rcp(double x) { return fx_rcp_ok(x) ? fx_rcp_normal(x) : fx_rcp_slow(x); }
+// a/b; a divisor without a normal reciprocal takes the division (1/b overflows where a/b need not)
+FX_SLOW double fx_div_slow(double a, double b) { return a / b; }
+FX_FN double fx_div(double a, double b) { return fx_rcp_ok(b) ? a * fx_rcp_normal(b) : fx_div_slow(a, b); }
 
 // exp(x): x in Q53 (exact; Q62 below 1) times log2(e), the product's integer part and 64 bits of its
 // fraction

@@ -1882,7 +1882,7 @@ __device__ double ros4_attempt(const Team& tm, double P, double hh, double rtol,
     tm.at(OFF_YT, i) = yn;
     const double ay = fabs(y), an = fabs(yn);
     const double sc = atol + rtol * (ay > an ? ay : an);
-    const double z = e * fx_rcp(sc);
+    const double z = fx_div(e, sc);
     acc += z * z;
     if (!isfinite(yn)) bad = true;
   }
