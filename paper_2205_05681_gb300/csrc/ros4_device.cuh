@@ -2382,6 +2382,12 @@ __device__ __forceinline__ DD xlog10(DD a) { return mk(fx_log(a.v) * (1.0 / LN10
 __device__ __forceinline__ DD xdiv(DD a, DD b) { return a / b; }
 __device__ __forceinline__ DD xdiv(double a, DD b) { return a / b; }
 __device__ __forceinline__ DD xdiv(DD a, double b) { return a / b; }
+// a/b where b may be too small to have a reciprocal (rate constants)
+__device__ __forceinline__ double xdiv_wide(double a, double b) { return fx_div(a, b); }
+__device__ __forceinline__ DD xdiv_wide(DD a, DD b) {
+  const double q = fx_div(a.v, b.v);
+  return mk(q, fx_div(a.d - q * b.d, b.v));
+}
 __device__ __forceinline__ double vof(double a) { return a; }
 __device__ __forceinline__ double vof(DD a) { return a.v; }
 __device__ __forceinline__ double dof(double a) { return 0.0; }
@@ -2524,7 +2530,7 @@ OUTLINE void vjp(double P, const double* __restrict__ lnA_ext) {
     }
     if (kind >= LIND) {
       const S k0 = xexp(mk_lnA0[r] + mk_b0[r] * lnT - mk_th0[r] * invT);
-      S Pr = xdiv(k0 * M, kinf);
+      S Pr = xdiv_wide(k0 * M, kinf);
       bool floored = false;
       if (vof(Pr) < 1e-300) { Pr = Z + 1e-300; floored = true; }
       S F = Z + 1.0, dlF_dlPr = Z, dlF_dT = Z;

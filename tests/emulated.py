@@ -68,6 +68,12 @@ EVAL = r"""
   ok = ok && emu::run(TPB, order, [&] { chem_eval_jacobian_k(n, T.data(), P.data(), X.data(), J.data(), n, lnA); });
   put(f); put(J);
 """
+# X: moles; then the weights v[k][cell]
+VJP = r"""
+  std::vector<double> v = arr((size_t)NS * n), gy(NS * n), gp(NR * n);
+  ok = emu::run(TPB, order, [&] { chem_eval_vjp_k(n, T.data(), P.data(), X.data(), v.data(), gy.data(), gp.data(), n, nullptr); });
+  put(gy); put(gp);
+"""
 # X: mass fractions Y[k][cell]; with argv[6] a cache of the W-method's factors
 INTEGRATE = r"""
   std::vector<double> h(n), C(WC_STRIDE * n);
@@ -112,6 +118,14 @@ class Emulated:
         X[:-1] = n.T
         o = self._run([order, c, int(lnA is not None)], [T, P, X, np.zeros(nr) if lnA is None else lnA])
         return o[:ns * c].reshape(ns, c).T, o[ns * c:].reshape(ns * ns, c).T.reshape(c, ns, ns)
+
+    def vjp(self, T, P, n, v, order=1):
+        """J^T v [cell, Ns] and (df/dlnA)^T v [cell, Nr]"""
+        c, ns = len(T), n.shape[1] + 1
+        X = np.zeros((ns, c))
+        X[:-1] = n.T
+        o = self._run([order, c], [T, P, X, v.T])
+        return o[:ns * c].reshape(ns, c).T, o[ns * c:].reshape(-1, c).T
 
     def integrate(self, T, P, Y, dt, rtol=1e-6, atol=1e-10, cache=False, order=1):
         """T, Y [cell, Ns], the factor cache, h, status and attempts"""
