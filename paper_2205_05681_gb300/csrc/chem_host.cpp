@@ -22,6 +22,7 @@
 #include <mutex>
 #include <sstream>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <tuple>
 #include <unordered_map>
@@ -1154,18 +1155,36 @@ int resolve(chem_mech* m, const chem_int_opts* o, Module** mod, int64_t n_cells 
   return get_module(m, team, tpb, mod, false, o ? o->tableau : 0);
 }
 
-// loads several configurations, compiling those that are not cached in parallel host threads
-// (NVRTC is thread-safe); the first must load, the others only if they fit
-int load_configs(chem_mech* m, const std::vector<std::pair<int, int>>& cfg, bool adjoint = false) {
+// cubins of several configurations, those that are not cached compiled in parallel host threads (NVRTC is
+// thread-safe); empty where that failed: get_module then says why.  Where no thread can be had
+// (a process at its limit) this one compiles, and nothing is thrown.
+std::vector<std::string> build_cubins(const chem_mech* m, const std::vector<std::pair<int, int>>& cfg, bool adjoint) {
   std::vector<std::string> cubins(cfg.size());
-  std::vector<std::thread> th;
-  for (size_t i = 0; i < cfg.size(); ++i)
-    th.emplace_back([&, i] {
+  auto one = [&](size_t i) {
+    try {
       std::string lg;
-      if (build_cubin(m->data, cfg[i].first, cfg[i].second, adjoint, 0, m->cache_dir.c_str(), m->verbose, &cubins[i], &lg))
-        cubins[i].clear();
-    });
+      if (!build_cubin(m->data, cfg[i].first, cfg[i].second, adjoint, 0, m->cache_dir.c_str(), m->verbose, &cubins[i], &lg))
+        return;
+    } catch (...) {
+    }
+    cubins[i].clear();
+  };
+  std::vector<std::thread> th;
+  th.reserve(cfg.size());
+  for (size_t i = 0; i < cfg.size(); ++i) {
+    try {
+      th.emplace_back(one, i);
+    } catch (const std::system_error&) {
+      one(i);
+    }
+  }
   for (auto& t : th) t.join();
+  return cubins;
+}
+
+// loads several configurations; the first must load, the others only if they fit
+int load_configs(chem_mech* m, const std::vector<std::pair<int, int>>& cfg, bool adjoint = false) {
+  const std::vector<std::string> cubins = build_cubins(m, cfg, adjoint);
   for (size_t i = 0; i < cfg.size(); ++i) {
     Module* mod;
     const int rc = get_module(m, cfg[i].first, cfg[i].second, &mod, adjoint, 0, &cubins[i]);
