@@ -50,16 +50,15 @@ METHODS = ["ROS4", "ROS3", "RODAS3", "RODAS4", "RKF45", "ROS2W"]
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one chem_integrate_k launch on the
 # full bench workload, from a single-pass ncu capture; valid only for the device source they were
-# taken on (sha1 of csrc/ros4_device.cuh), reported as null once that source changes.
+# taken on (sha1 of csrc/fxmath.cuh followed by csrc/ros4_device.cuh), reported as null once it changes.
 MEASURED_TRAFFIC = {"device_src_sha1": "4ff7f10b7da918bc04f1b55c6db25a30a4a18cc9",
                     "ch4_111_batched": 250775808 + 204967680}
 
 
 def measured_traffic(wl, full_size):
     import hashlib
-    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2205_05681_gb300",
-                       "csrc", "ros4_device.cuh")
-    sha = hashlib.sha1(open(src, "rb").read()).hexdigest()
+    from paper_2205_05681_gb300 import build
+    sha = hashlib.sha1(b"".join(open(p, "rb").read() for p in build.DEVICE)).hexdigest()
     if not full_size or sha != MEASURED_TRAFFIC["device_src_sha1"]:
         return None
     return MEASURED_TRAFFIC.get(wl)
