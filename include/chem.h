@@ -25,6 +25,12 @@
  *   - Calls are asynchronous on `stream` (a cudaStream_t; NULL = legacy default stream) and
  *     return once the work is enqueued.  chem_integrate in CHEM_MODE_PERSISTENT does no host
  *     synchronisation and no allocation, so it can be captured in a CUDA graph.
+ *   - The lanes per cell set the order of a cell's sums.  Without a configuration (chem_build_opts,
+ *     chem_int_opts or chem_autotune) they follow the call's number of cells, so a cell's result may
+ *     differ in rounding, and by an accept/reject decision that hangs on it, between calls of
+ *     different sizes; ask for a configuration where a batch is split over calls or ranks and has
+ *     to give the same.  Two runs of one call differ in rounding too: third-body and falloff terms
+ *     of the Jacobian are added by atomics in no fixed order.
  *   - Return value: 0 on success, negative on an argument, CUDA or NVRTC error; the message is
  *     in chem_last_error() (thread-local).  Integration failures of single cells are never
  *     errors: they are reported per cell in `status`.

@@ -1037,6 +1037,17 @@ std::vector<std::pair<int, int>> size_configs(int ns, bool adjoint = false) {
 // so the lines lie at 12 and 160 cells per SM (13 species) and at 4, a resident team of 128 lanes
 // each (53 species).  One evaluation of f or J (eval): the same lines for 13 species (50,000 cells, source
 // 0.20 ms at 8 lanes and 0.56 at 64); at 53 species 64 lanes win from 1,000 cells on.
+// Between and beside them (the same split step, ms):
+//   lanes                 8      16      64        lanes                64     128
+//   14 sp,  1,000 cells 1.93    1.21    1.10       24 sp,   300 cells  12.6    11.1
+//           5,000       2.47    2.01    2.87                 1,200     14.4    20.0
+//          40,000       7.96    8.55    19.5       36 sp,   300        11.4    10.0
+//   16 sp,  1,000       2.28    1.53    1.12                 1,200     16.7    18.9
+//           5,000       2.88    2.52    3.00       46 sp,   600        20.6    17.3
+//          40,000       10.1    10.9    20.6       17 sp,   300        1.10    1.18
+//   17 sp, 40,000       10.4    12.1    22.5       20 sp,   600        1.34    1.47
+// so the classes end too low: 8 lanes would serve large batches of 17 to 20 species too, and 128 cost few
+// cells of these 2 to 9%.
 enum CallKind { kIntegrate, kEval, kAdjoint };
 void config_for(int ns, int64_t n, int n_sm, CallKind kind, int* team, int* tpb) {
   if (ns <= 16) {

@@ -3,7 +3,7 @@
 // GB300 issues an FP64 instruction per 16 clocks and SM (64 clocks of latency); a 64-bit integer
 // multiply (umul64hi, about six IMADs) takes 5 clocks of an SM and 41 of latency.  A CUDA exp()
 // occupies an SM for 304 clocks, log() for 568 and a division for 86 (latencies 1087, 2088 and
-// 380; measured with all warps busy and with one warp).  The functions below keep 62 or more
+// 380; measured with all warps busy and with one warp).  The functions below keep 58 or more
 // correct bits in 64-bit fixed point, use no FP64 instruction, and round once to a double.
 //
 // Fixed-point formats are written Qn: an integer v stands for v 2^-n.
@@ -107,7 +107,8 @@ FX_FN double fx_exp2_nf(int n, fx_u64 F) {
 }
 FX_FN double fx_exp2(fx_i64 lg) { return fx_exp2_nf((int)(lg >> 52), (fx_u64)lg << 12); }
 
-// log2 of the 53-bit mantissa m in [2^52, 2^53): Q62, in [0, 1] up to 2^-60
+// log2 of the 53-bit mantissa m in [2^52, 2^53): Q62, in [0, 1], off by 2.2 2^-59 at most (the 32-bit tail of
+// the series)
 FX_FN fx_i64 fx_log2_mant(fx_u64 m) {
   const int i = (int)(m >> 46) & 63;
   const fx_i64 z = (fx_i64)(m * fx_t_rcp[i] - (1ULL << 62)) << 7;  // 2^7 z, Q62
